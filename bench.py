@@ -483,9 +483,12 @@ def config2_step(dev, flush, stream, steps=5):
 # source files each bounding kernel is built from (the traffic record is valid
 # only while they are unchanged)
 KERNEL_SOURCES = {
-    "interpreter": ("ivb_kernels.cu", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fp64x.cuh", "ivb_emu.cuh"),
-    "specialised": ("ivb_jit.cpp", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fp64x.cuh", "ivb_emu.cuh"),
-    "segmented": ("ivb_jit_seg.cpp", "ivb_jit.h", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fp64x.cuh", "ivb_emu.cuh"),
+    "interpreter": ("ivb_kernels.cu", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fixed.cuh", "ivb_fp64x.cuh",
+                    "ivb_emu.cuh"),
+    "specialised": ("ivb_jit.cpp", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fixed.cuh", "ivb_fp64x.cuh",
+                    "ivb_emu.cuh"),
+    "segmented": ("ivb_jit_seg.cpp", "ivb_jit.h", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fixed.cuh", "ivb_fp64x.cuh",
+                    "ivb_emu.cuh"),
 }
 
 

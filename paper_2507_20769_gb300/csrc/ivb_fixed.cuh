@@ -1,0 +1,198 @@
+// ivb_fixed.cuh -- reciprocal, quotient, square root, exp and log with directed
+// rounding, on 64-bit fixed-point integers: no FP64 instruction.
+//
+// GB300's FP64 pipe takes one warp instruction per 64 cycles of an SM
+// sub-partition (76 when all four are busy), while a 32 x 32 -> 64 bit
+// multiply-add costs 5 and a 64-bit high product 17. With FP64 refinement
+// steps these five functions were half of all FP64 instructions of the
+// bounding kernels (4 per quotient end, 2 to 3 per reciprocal, 5 per root and
+// exp, 8 per log); in fixed point an end costs 35 to 80 integer instructions,
+// about as many as the bit assembly around the FP64 steps took.
+//
+// Reciprocal, quotient and root: Newton steps from a 23-bit MUFU seed
+// (Markstein's method, IBM J. Res. Dev. 34, 1990, in integers) give the
+// significand with an error in (0, 1) units of the last place, upwards; the
+// sign of the exact remainder, read from the low 64 bits of a product, then
+// decides whether the directed result is this significand or its neighbour.
+// The remainder is 0 for exact results, and a step across a power of two is a
+// carry into the exponent, so the fast path covers every normal result.
+//
+// exp and log: Tang's table-driven method (ACM TOMS 15(2) 1989 and 16(4)
+// 1990), arguments reduced modulo 1 in units of 2^-64. The sums of all
+// truncations are within (-13.5, 1.5) units of 2^-62 (exp, of a significand in
+// [1, 2)) and (-12.1, 8.4) units of 2^-64 (log); each end is moved outward by that
+// before it is rounded outward: 1 step from the true value, 2 in about one
+// case of 100.
+//
+// Plain C++ but for the intrinsics __umulhi, __mulhi, __clz and
+// __funnelshift_l, bits(), from_bits() and the two MUFU approximations: the
+// CPU tests compile this file with stand-ins for them.
+#pragma once
+
+namespace ivb {
+
+typedef unsigned int fx32;
+typedef unsigned long long fx64;
+
+constexpr int kExpTab = 512, kLogTab = 1024;
+struct LogEntry {          // c_j = c 2^-20 just above 1 / (1 + j / 1024)
+    fx32 c;
+    int ip;                // -log(c_j) - 1023 ln2 = ip + frac 2^-64
+    fx64 frac;
+};
+
+__device__ __forceinline__ fx32 lo32(fx64 v) { return (fx32)v; }
+__device__ __forceinline__ fx32 hi32(fx64 v) { return (fx32)(v >> 32); }
+__device__ __forceinline__ fx64 join(fx32 hi, fx32 lo) { return ((fx64)hi << 32) | lo; }
+__device__ __forceinline__ fx64 wide(fx32 a, fx32 b) { return (fx64)a * b; }
+
+// significand of a normal double as the integer in [2^52, 2^53)
+__device__ __forceinline__ fx64 sig53(double x) {
+    return ((fx64)bits(x) & 0x000FFFFFFFFFFFFFULL) | 0x0010000000000000ULL;
+}
+// top 23 bits after the leading one of a significand, as the float in [1, 2)
+__device__ __forceinline__ int top23(fx64 Y) { return (int)((fx32)(Y >> 29) & 0x7FFFFFu); }
+// 24-bit integer of a float in [0.5, 1], in units of 2^-24
+__device__ __forceinline__ fx32 unit24(float r) { return (fx32)(__float_as_int(r) - 0x3E800000); }
+
+// 2^52 / Y in units of 2^-62, too large by 3 to 10 units. With
+// e = 1 - Y R0 / 2^76 of the seed (|e| < 2^-21.6; Y R0 modulo 2^64 is -e 2^76),
+// R0 (1 + e + e^2) leaves e^3 < 2^-64.
+__device__ __forceinline__ fx64 rcp62(fx64 Y) {
+    const fx32 R0 = unit24(rcp_approx_f(__int_as_float(0x3F800000 | top23(Y))));
+    const long long e = -(long long)(Y * R0);              // 2^-76, below 2^54.4
+    const int eh = (int)(e >> 32);
+    const long long u = e + ((long long)eh * eh >> 12);    // e + e^2
+    const long long p = (long long)(int)(u >> 32) * (long long)R0 + (long long)hi32(wide(lo32(u), R0));
+    return ((fx64)R0 << 38) + (fx64)(p >> 6) + 6;
+}
+
+// round the significand q 2^k, too large by less than one unit, of the value
+// whose remainder has the sign of rem (rem < 0: q is above the value)
+__device__ __forceinline__ fx64 settle(fx64 q, long long rem, bool away) {
+    return away ? q + (rem > 0 ? 1 : 0) : q - (rem < 0 ? 1 : 0);
+}
+
+__device__ __forceinline__ int bexp(double x) { return (int)((bits(x) >> 52) & 0x7FF); }
+
+// 1 / |y| for y normal with a normal reciprocal; away: toward +inf
+__device__ __forceinline__ bool rcp_fits(double y) { return (fx32)(bexp(y) - 1) < 2044u; }
+__device__ __forceinline__ fx64 rcp_mag(double y, bool away) {
+    const fx64 Y = sig53(y);
+    const fx64 q = rcp62(Y) >> 9;                          // units of 2^-53
+    const long long rem = -(long long)(Y * q);             // 2^105 - Y q
+    return settle(q, rem, away) + ((fx64)(fx32)(2044 - bexp(y)) << 52);
+}
+
+// |x| / |y| for normal x and y with |Ex - Ey| <= 1000; r62 = rcp62(sig53(y))
+__device__ __forceinline__ bool div_fits(double x, double y) {
+    const int Ex = bexp(x), Ey = bexp(y);
+    return (fx32)(Ex - 1) < 2046u && (fx32)(Ey - 1) < 2046u && (fx32)(Ex - Ey + 1000) <= 2000u;
+}
+// high 64 bits of a product, at most 2 below it: the product of the low words is left out
+__device__ __forceinline__ fx64 mulhi64_near(fx64 a, fx64 b) {
+    const fx64 m = wide(hi32(a), lo32(b)), n = wide(lo32(a), hi32(b));
+    return wide(hi32(a), hi32(b)) + hi32(m) + hi32(n);
+}
+__device__ __forceinline__ fx64 div_mag(double x, double y, fx64 r62, bool away) {
+    const fx64 X = sig53(x), Y = sig53(y);
+    const fx64 h = mulhi64_near(X << 11, r62 + 4);         // x / y in units of 2^-61, too large by 1 to 14
+    const int big = (int)(h >> 61);                        // quotient >= 1
+    const fx64 q = h >> (8 + big);
+    const long long rem = (long long)((X << (53 - big)) - Y * q);
+    return settle(q, rem, away) + ((fx64)(fx32)(bexp(x) - bexp(y) + 1021 + big) << 52);
+}
+
+// sqrt of a normal x > 0. g0 = a r0 (32 bits, r0 the seed cut below
+// 1/sqrt(a)), d = a - g0^2 exactly, then c = d r0 / 2 and the second order
+// c (eta - c r0 / 2) with eta = 1 - g0 r0; the third is below 2^-56.
+__device__ __forceinline__ bool sqrt_fits(double x) { return (fx32)((bits(x) >> 52) - 1) < 2046u; }
+__device__ __forceinline__ fx64 sqrt_mag(double x, bool up) {
+    const int E = bexp(x), odd = (E + 1) & 1;
+    const fx64 Y = sig53(x), A = Y << odd;                 // a in [1, 4) in units of 2^-52
+    const fx32 R0 = unit24(rsqrt_approx_f(__int_as_float(((127 + odd) << 23) | top23(Y)))) - 4;
+    const fx64 ar = wide(hi32(A), R0) + __umulhi(lo32(A), R0);   // a r0, 2^-44
+    const fx32 G = (fx32)(ar >> 13);                       // 2^-31
+    const fx64 d = (A << 10) - wide(G, G);                 // 2^-62, below 2^44
+    const fx64 c = ((d >> 8) * R0) >> 17;                  // 2^-62
+    const fx32 eta = (fx32)((((fx64)1 << 55) - wide(G, R0)) >> 8);   // 2^-47
+    const fx32 cq = (fx32)(c >> 14);                       // 2^-48
+    const fx32 w = eta - (__umulhi(cq, R0 << 7) >> 1);     // eta - c r0 / 2, 2^-47
+    const fx64 s = ((fx64)G << 31) + c + (__umulhi(cq, w) >> 1) + 512;   // 2^-62
+    const fx64 q = s >> 10;
+    const long long rem = (long long)((A << 52) - q * q);
+    return settle(q, rem, up) + ((fx64)(fx32)((E - 1023 - odd) / 2 + 1022) << 52);
+}
+
+// exp(x) rounded outward, |x| <= 700. With L = ln2 / 512 and k = floor(x / L)
+// (at most 0.004 below it): exp(x) = 2^(k / 512) e^r, r = x - k L in [0, 1.004 L);
+// e^r - 1 = r + r^2/2 (1 + r (1/3 + r/12 + r^2/60)). x modulo 1 and k L modulo 1 are
+// integers in units of 2^-64, so r comes out of one subtraction.
+__device__ __forceinline__ bool exp_fits(double x) {
+    return (fx32)hi32((fx64)bits(x) & 0x7FFFFFFFFFFFFFFFULL) < 0x4085E000u;   // |x| < 700
+}
+__device__ __forceinline__ fx64 exp_mag(double x, const fx64* __restrict__ tab, bool up) {
+    const int E = bexp(x);
+    const long long neg = bits(x) >> 63;                   // 0 or -1
+    const fx64 B = sig53(x) << 11;
+    const int l = E >= 1022 ? E - 1022 : 0, r0 = E >= 1022 ? 0 : (E < 959 ? 63 : 1022 - E);
+    const fx64 X = (B << l) >> r0;                         // |x| modulo 1
+    const int sh = 1033 - E;
+    const int x21 = (int)((sh < 32 ? hi32(B) >> sh : 0u) ^ (fx32)neg);        // x in units of 2^-21, rounded down
+    const fx32 k = (fx32)(__mulhi(x21, 1549082004) + (1 << 30) - 1) >> 10;    // floor(x / L) + 2^20
+    const fx64 kL = ((fx64)(k * 0x0058B90Bu) << 32) + wide(k, 0xFBE8E7BCu) + __umulhi(k, 0xD5E4F1D9u);
+    const fx64 r = (X ^ (fx64)neg) - kL + 0x90BFBE8E7BCD5E4FULL;              // + 2^20 L
+    const fx32 rq = (fx32)(r >> 23);                       // 2^-41
+    const fx64 h = (wide(rq, rq) >> 19) + __umulhi(rq, (lo32(r) >> 9) & 0x3FFFu);   // r^2 / 2
+    const fx32 rh = hi32(r);
+    const fx32 w = 0x55555555u + __umulhi(rh, 0x15555555u + __umulhi(rh, 0x04444444u));
+    const fx64 tail = wide((fx32)(h >> 12), __umulhi(rq, w)) >> 29;
+    const fx64 p = r + h + tail;
+    const fx64 T = tab[k & (kExpTab - 1)];                 // 2^(j / 512) in units of 2^-62
+    const fx32 cross = __umulhi(hi32(T), lo32(p)) + __umulhi(lo32(T), hi32(p));
+    const fx64 M = T + wide(hi32(T), hi32(p)) + cross + (up ? 14 : -2LL);
+    const int top = (int)(M >> 63);
+    return (M >> (10 + top)) + ((fx64)(fx32)((int)(k >> 9) - 2048 + 1022 + top) << 52) + (up ? 1 : 0);
+}
+
+// log(x) rounded outward for a normal x > 0, or 0 (false) where |log x| is
+// below 2^-7: units of 2^-64 are too coarse there. x = 2^m y, y c_j = 1 + r with
+// 0 <= r < 2^-9.99 exact in 64 bits; log1p(r) = r - r^2/2 (1 - r (2/3 - r/2 + 2 r^2/5)).
+__device__ __forceinline__ bool log_fits(double x) { return (fx32)((bits(x) >> 52) - 1) < 2046u; }
+__device__ __forceinline__ bool log_val(double x, const LogEntry* __restrict__ tab, bool up, double* out) {
+    const fx32 E = (fx32)bexp(x);
+    const fx64 Y = sig53(x);
+    const LogEntry T = tab[(hi32(Y) >> 10) & (kLogTab - 1)];
+    const fx64 r = (Y * T.c) >> 8;                         // y c_j - 1
+    const fx32 rq = (fx32)(r >> 23), rh = hi32(r);
+    const fx64 h = (wide(rq, rq) >> 19) + __umulhi(rq, (lo32(r) >> 9) & 0x3FFFu);
+    const fx32 w = 0xAAAAAAABu - __umulhi(rh, 0x80000000u - __umulhi(rh, 0x66666666u));
+    const fx64 tail = wide((fx32)(h >> 12), __umulhi(rq, w)) >> 29;
+    const fx64 l1p = r - h + tail;
+    // E ln2 + (-log c_j - 1023 ln2) + log1p(r): integer word and 64 bits of fraction
+    const fx64 a = wide(E, 0xD1CF79ABu) + __umulhi(E, 0xC9E3B398u);
+    const fx64 b = wide(E, 0xB17217F7u) + hi32(a);
+    fx64 f = join(lo32(b), lo32(a));
+    fx32 ip = hi32(b) + (fx32)T.ip;
+    f += T.frac;
+    ip += f < T.frac ? 1u : 0u;
+    f += l1p;
+    ip += f < l1p ? 1u : 0u;
+    const bool neg = (int)ip < 0;
+    const fx32 s = neg ? ~0u : 0u;
+    ip ^= s;
+    f ^= join(s, s);
+    if (ip == 0u && hi32(f) < 0x02000000u) return false;
+    const bool away = up != neg;
+    const fx64 g = away ? f + 13 : f - 13;
+    ip += away ? (g < f ? 1u : 0u) : (g > f ? ~0u : 0u);
+    const bool small = ip == 0u;
+    const fx32 w2 = small ? hi32(g) : ip, w1 = small ? lo32(g) : hi32(g), w0 = small ? 0u : lo32(g);
+    const int lz = __clz((int)w2);
+    const fx64 mant = join(__funnelshift_l(w1, w2, lz), __funnelshift_l(w0, w1, lz));
+    const fx64 m = (mant >> 11) + ((fx64)(fx32)((small ? 1021 : 1053) - lz) << 52) + (away ? 1 : 0);
+    *out = from_bits((long long)(m | (neg ? 0x8000000000000000ULL : 0ULL)));
+    return true;
+}
+
+}  // namespace ivb

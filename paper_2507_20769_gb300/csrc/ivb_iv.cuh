@@ -3,8 +3,8 @@
 // Natural interval extensions of the intrinsics (Section 2.2) with directed
 // rounding from the CUDA rounding-mode intrinsics (__dadd_rd / __dmul_ru /
 // __ddiv_rd / __dsqrt_ru / __drcp_rd ...; Section 3.2 notes that basic
-// operations support all rounding modes on the GPU), and two-ulp outward
-// widening of exp/log, whose documented error is one ulp.
+// operations support all rounding modes on the GPU); quotients, reciprocals and
+// roots correctly rounded in fixed point, exp and log rounded outward there.
 //
 // GB300 has a narrow FP64 pipe (one warp instruction per 64 cycles per SM
 // sub-partition) while the integer pipes are wide, so everything that is not
@@ -249,7 +249,7 @@ __device__ __forceinline__ iv iv_sqr(iv x) { return iv_sqr_t<IVB_EMU>(x); }
 // reciprocal of an interval without 0 (ENTIRE otherwise)
 __device__ IVB_HEAVY iv iv_recip(iv y) {
     if (!(gt0(y.lo) || lt0(y.hi))) return entire();
-    return mk(rcp_dn(y.hi), rcp_up(y.lo));
+    return mk(rcp_dir(y.hi, false), rcp_dir(y.lo, true));
 }
 __device__ __forceinline__ iv iv_recip_pos(iv y) { return gt0(y.lo) ? iv_recip(y) : entire(); }
 
@@ -257,14 +257,12 @@ __device__ __forceinline__ iv iv_recip_pos(iv y) { return gt0(y.lo) ? iv_recip(y
 __device__ IVB_HEAVY iv iv_div(iv x, iv y) {
     const bool ypos = gt0(y.lo), yneg = lt0(y.hi);
     if (!(ypos || yneg) || has_inf(x) || has_inf(y)) return entire();
-    // for y < 0 use x/y = (-x)/(-y) with -y > 0 (negations are exact)
-    double xl = x.lo, xh = x.hi, yl = y.lo, yh = y.hi;
-    if (yneg) { xl = ineg(x.hi); xh = ineg(x.lo); yl = ineg(y.hi); yh = ineg(y.lo); }
-    const double dl = ge0(xl) ? yh : yl;
-    const double dh = ge0(xh) ? yl : yh;
-    const double rl = rcp_refined(dl);
-    const double rh = (bits(dh) == bits(dl)) ? rl : rcp_refined(dh);
-    return mk(div_dir_pos(xl, dl, rl, false), div_dir_pos(xh, dh, rh, true));
+    // numerators of the two ends; a quotient >= 0 is least (most) over the
+    // divisor of largest (smallest) magnitude, one < 0 the other way round
+    const double nl = yneg ? x.hi : x.lo, nh = yneg ? x.lo : x.hi;
+    const double dl = (yneg ? le0(nl) : ge0(nl)) != yneg ? y.hi : y.lo;
+    const double dh = (yneg ? le0(nh) : ge0(nh)) != yneg ? y.lo : y.hi;
+    return mk(div_dir(nl, dl, false), div_dir(nh, dh, true));
 }
 
 __device__ IVB_HEAVY iv iv_sqrt(iv x) {
@@ -272,20 +270,15 @@ __device__ IVB_HEAVY iv iv_sqrt(iv x) {
     return mk(sqrt_dir(x.lo, false), sqrt_dir(x.hi, true));
 }
 
-// exp / log: table-driven evaluation (ivb_fp64x.cuh) widened two neighbour
-// steps outward; the lower end of exp is clamped at 0.
+// exp / log rounded outward (ivb_fp64x.cuh); the lower end of exp is clamped at 0
 __device__ __forceinline__ double exp_dn(double x) {
     double r = exp_dir(x, false);
     return lt0(r) ? 0.0 : r;
 }
-__device__ __forceinline__ double exp_up(double x) { return exp_dir(x, true); }
-__device__ __forceinline__ double log_dn(double x) { return log_dir(x, false); }
-__device__ __forceinline__ double log_up(double x) { return log_dir(x, true); }
-
-__device__ IVB_HEAVY iv iv_exp(iv x) { return mk(exp_dn(x.lo), exp_up(x.hi)); }
+__device__ IVB_HEAVY iv iv_exp(iv x) { return mk(exp_dn(x.lo), exp_dir(x.hi, true)); }
 __device__ IVB_HEAVY iv iv_log(iv x) {
     if (!gt0(x.lo)) return entire();
-    return mk(log_dn(x.lo), log_up(x.hi));
+    return mk(log_dir(x.lo, false), log_dir(x.hi, true));
 }
 
 // intersection of two enclosures of the same quantity

@@ -530,8 +530,8 @@ __global__ void k_own_probe(double* out, double seed, int iters) {
         const double d = (i & 1) ? 0.0009765625 : -0.0009765625;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            if (W == 0) x[j] = rcp_dir_pos(x[j], false);
-            if (W == 1) x[j] = div_dir_pos(y, x[j], rcp_refined(x[j]), false);
+            if (W == 0) x[j] = rcp_dir(x[j], false);
+            if (W == 1) x[j] = div_dir(y, x[j], false);
             if (W == 2) x[j] = sqrt_dir(x[j] * 3.1, false);   // one multiply keeps x off powers of two
             if (W == 3) x[j] = exp_dir(-x[j], false);
             if (W == 4) x[j] = __dadd_rn(log_dir(x[j], false), 2.0);
@@ -581,8 +581,7 @@ cudaError_t run_own_probe(int which, double* out, int grid, int block, int iters
 }
 
 // exp/log tables in extended precision on the host (long double: 64-bit
-// significand on x86-64, binary128 on AArch64), split into double hi + lo
-// (the exp table keeps hi, and hi and lo rounded to float)
+// significand on x86-64, binary128 on AArch64)
 cudaError_t math_tables_address(void** ptr, size_t* bytes) {
     *bytes = sizeof(MathTables);
     return cudaGetSymbolAddress(ptr, g_math);
@@ -595,26 +594,26 @@ cudaError_t init_math_tables() {
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 256 && done[dev]) return cudaSuccess;
     static MathTables h;
-    for (int j = 0; j < kExpTab; ++j) {
-        const long double v = exp2l((long double)j / kExpTab);
-        h.exp[j].hi = (double)v;
-        h.exp[j].hi_f = (float)h.exp[j].hi;
-        h.exp[j].lo_f = (float)(v - (long double)h.exp[j].hi);
-    }
-    const long double T = kLogTab;
+    const long double two32 = 4294967296.0L;
+    for (int j = 0; j < kExpTab; ++j)
+        h.exp[j] = (fx64)(exp2l((long double)j / kExpTab) * (two32 * (two32 / 4)) + 0.5L);
+    // 1023 ln2 = 710 - frac 2^-64
+    const fx64 frac = 0xE91238B093E8CA84ULL;
     for (int j = 0; j < kLogTab; ++j) {
-        // y in [1 + j/T, 1 + (j+1)/T); the upper half is folded to y/2 in [0.75, 1);
+        h.log[j].c = (fx32)(((1u << 30) + (kLogTab + j) - 1) / (kLogTab + j));
+        const fx64 v = (fx64)(-logl((long double)h.log[j].c / 1048576.0L) * (two32 * two32) + 0.5L);
+        h.log[j].frac = v + frac;
+        h.log[j].ip = -710 + (h.log[j].frac < v ? 1 : 0);
+    }
+    for (int k = 0; k < kNearTab; ++k) {
         // the two intervals next to 1 use c = 1 so that r = y - 1 is exact
-        double c = 1.0;
-        if (j != 0 && j != kLogTab - 1) {
-            const long double F = (j < kLogTab / 2) ? 1.0L + (j + 0.5L) / T : (1.0L + (j + 0.5L) / T) / 2.0L;
-            c = (double)(1.0L / F);
-        }
+        const int j = k - kNearTab / 2;
+        const long double F = j >= 0 ? 1.0L + (j + 0.5L) / 2048 : (1.0L + (2048 + j + 0.5L) / 2048) / 2;
+        const double c = j == 0 || j == -1 ? 1.0 : (double)(1.0L / F);
         const long double L = -logl((long double)c);
-        h.log[j].c = c;
-        h.log[j].hi = (double)L;
-        h.log[j].lo = (double)(L - (long double)h.log[j].hi);
-        h.log[j].pad = 0.0;
+        h.near1[k].c = c;
+        h.near1[k].hi = (double)L;
+        h.near1[k].lo = (double)(L - (long double)h.near1[k].hi);
     }
     e = cudaMemcpyToSymbol(g_math, &h, sizeof(h));
     if (e == cudaSuccess && dev >= 0 && dev < 256) done[dev] = true;
