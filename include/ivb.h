@@ -127,10 +127,11 @@ typedef struct {
                                   mode only; for large tapes);
                                   0 (default): tape interpreter; -1: as 1 when
                                   the tape has at most 1024 interval
-                                  operations per subdomain, else as 3 in
-                                  adjoint mode and the interpreter in forward
-                                  mode, and the autotuner keeps the
-                                  interpreter instead when it times faster  */
+                                  operations per subdomain (256 in adjoint
+                                  mode), else as 3 in adjoint mode and the
+                                  interpreter in forward mode, and the
+                                  autotuner keeps the interpreter instead
+                                  when it times faster                      */
     int32_t emulate;           /* tape-specialised kernel only: endpoint
                                   operations computed by an exact emulation
                                   on the integer pipes (bit-identical to the
@@ -153,7 +154,7 @@ typedef struct {
     int32_t seg_chunk;         /* segmented kernel: estimated FP64 issue
                                   slots per chunk (0 = default 320)         */
     int32_t seg_regs;          /* segmented kernel: register budget of every
-                                  chunk function, 64..255 (0 = default 128) */
+                                  chunk function, 64..255 (0 = default 64)  */
     int32_t threads_per_subdomain; /* segmented kernel with an own program
                                   per output: 1, 2 or 4 threads (in different
                                   warps of a block) share one subdomain, each
@@ -182,7 +183,7 @@ typedef struct {
                                   per statement); 2 only * sqr and the fused
                                   accumulation (+ and - inline); 0 inlines
                                   them all; -1 (default): the library's
-                                  choice, now 1                             */
+                                  choice, now 2                             */
 } ivb_options;
 
 typedef struct ivb_problem ivb_problem;

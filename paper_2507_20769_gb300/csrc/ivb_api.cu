@@ -257,7 +257,7 @@ std::vector<bool> sync_choices(const ivb_problem* p) {
 // times larger grabs (4 and 16 passes per grab) for the best of stage 1.
 ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
     std::vector<TuneCand> cands;
-    const int blocks[] = {64, 128, 256};
+    const int blocks[] = {1024, 512, 64, 128, 256};   // above 256: segmented kernels only
     const int bpss[] = {1, 2, 3, 4, 6, 8};
     int max_threads = 0;
     // with the library's choice of kernel, the interpreter competes with the
@@ -273,6 +273,7 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
             for (int k : bpss) {
                 const int warps = b * k / 32;
                 if (warps < 4 || warps > 32 || b < 32 * t) continue;
+                if (b > 256 && !(reduce_jit(p) && p->jit.state_units > 0 && b <= p->jit.block_max)) continue;
                 for (int sm = 0; sm < 2; ++sm) {
                     const size_t bytes = smem_bytes(p, b, sm);
                     if (sm && (reduce_jit(p) || bytes + 1024 > (size_t)p->smem_optin || bytes * k > 220 * 1024)) continue;
@@ -368,8 +369,12 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
 }
 
 ivb_status default_tuning(ivb_problem* p) {
-    p->block = p->opt.block_threads > 0 ? p->opt.block_threads : 128;
-    p->bps = p->opt.blocks_per_sm > 0 ? p->opt.blocks_per_sm : 4;
+    // a segmented kernel runs best as one block per SM: its warps then stream
+    // through the same code (configuration 5, 2^19 subdomains: 1024-thread
+    // blocks 56 ms, 2 x 512 71 ms, 4 x 256 118 ms)
+    const bool seg = reduce_jit(p) && p->jit.state_units > 0;
+    p->block = p->opt.block_threads > 0 ? p->opt.block_threads : seg ? p->jit.block_max : 128;
+    p->bps = p->opt.blocks_per_sm > 0 ? p->opt.blocks_per_sm : seg && p->opt.block_threads <= 0 ? 1 : 4;
     const size_t bytes = smem_bytes(p, p->block, 1);
     if (reduce_jit(p)) p->frame_smem = 0;   // frames serve only the interpreter's store mode
     else if (p->opt.frame_in_shared == 1) p->frame_smem = 1;
@@ -377,7 +382,8 @@ ivb_status default_tuning(ivb_problem* p) {
     else p->frame_smem = (bytes + 1024 <= (size_t)p->smem_optin && bytes * p->bps <= 220 * 1024) ? 1 : 0;
     p->tpsub = tpsub_choices(p).front();
     if (p->block < 32 * p->tpsub) p->tpsub = 1;
-    p->chunk_sync = sync_choices(p).front();
+    // code larger than the instruction caches: keep the warps on one chunk
+    p->chunk_sync = seg && p->jit.chunks >= kSegSyncChunks ? sync_choices(p).back() : sync_choices(p).front();
     const int occ = reduce_occupancy(p, p->block, p->frame_smem, p->tpsub, p->chunk_sync);
     if (occ < 1) return fail(p, IVB_ENOTSUP, "launch configuration does not fit on an SM");
     if (p->bps > occ) p->bps = occ;
@@ -420,22 +426,23 @@ SegPolicy seg_policy(const ivb_options& o) {
     if (o.recompute >= 0) pol.recompute = o.recompute;
     if (o.seg_chunk > 0) pol.chunk_cost = o.seg_chunk;
     if (o.seg_ilp > 0) pol.ilp = o.seg_ilp;
-    pol.outline = o.seg_outline < 0 ? 1 : o.seg_outline;   // -1: the library's choice, all out of line
+    if (o.seg_outline >= 0) pol.outline = o.seg_outline;
     if (o.seg_regs > 0) pol.max_regs = o.seg_regs;
     const unsigned hc = std::thread::hardware_concurrency();
     pol.units = std::max(1, std::min(64, hc ? (int)hc : 8));
     return pol;
 }
 
-// blocks of kJitBlockMax threads per SM that a register budget allows
-int seg_min_blocks(int max_regs) { return std::max(1, std::min(8, 65536 / (kJitBlockMax * max_regs))); }
+// threads of the largest block of a segmented kernel: all that a register
+// budget allows on an SM, in whole groups of four warps
+int seg_block_max(int max_regs) { return std::min(1024, 65536 / max_regs / 128 * 128); }
 
 cudaError_t specialize_seg(ivb_problem* p, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
                            const std::vector<double>& consts, std::string* msg) {
     const int emu = p->opt.emulate >= 0 ? p->opt.emulate : kJitDefaultEmulate;
     const SegPolicy pol = seg_policy(p->opt);
-    const SegSource src = jit_seg_source(p->P, ins, rins, consts, kJitBlockMax, seg_min_blocks(pol.max_regs), emu,
-                                         p->opt.form, pol);
+    const int block_max = seg_block_max(pol.max_regs);
+    const SegSource src = jit_seg_source(p->P, ins, rins, consts, block_max, emu, p->opt.form, pol);
     std::vector<char> cubin;
     std::string tables;
     double secs = 0.0;
@@ -456,7 +463,7 @@ cudaError_t specialize_seg(ivb_problem* p, const std::vector<Ins>& ins, const st
     p->jit.mode = KM_ADJ_REDUCE;
     p->jit.emulate = emu;
     p->jit.compact = true;
-    p->jit.block_max = kJitBlockMax;
+    p->jit.block_max = block_max;
     p->jit.compile_seconds = secs;
     p->jit.state_units = src.state_units;
     p->jit.chunks = src.chunks;
@@ -626,7 +633,7 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
         const int64_t* cnt = o.grad_mode == IVB_GRAD_ADJOINT ? p->P.cnt_adj : p->P.cnt_fwd;
         long long ops = 0;
         for (int k = 0; k < IVB_CNT_N; ++k) ops += cnt[k];
-        const bool small = ops / 2 <= kJitAutoMaxOps;
+        const bool small = ops / 2 <= (o.grad_mode == IVB_GRAD_ADJOINT ? kSegMinOps : kJitAutoMaxOps);
         const bool seg = o.specialize == 3 || (o.specialize == -1 && !small && o.grad_mode == IVB_GRAD_ADJOINT);
         if (o.specialize >= 1 || small || seg) {
             const int mode = o.grad_mode == IVB_GRAD_ADJOINT ? KM_ADJ_REDUCE : KM_FWD_REDUCE;
@@ -798,18 +805,21 @@ extern "C" ivb_status ivb_enclose(ivb_problem* p, const double* box, const int32
     if (out_G && !dG) CK(cudaMallocAsync(&tG, gb, s));
     const unsigned long long first_u = (unsigned long long)first;
     CK(cudaMemcpyAsync(p->d_counter, &first_u, sizeof(first_u), cudaMemcpyHostToDevice, s));
-    const long long tiles = (count + p->block - 1) / p->block;
-    const int grid = (int)std::min<long long>(tiles, (long long)p->sm_count * p->bps);
-    st = ensure_frame(p, grid, p->block, frame_units(p));
+    // the store modes run the interpreter: its own shape when the reduce launches use another kernel
+    const bool own = !reduce_jit(p);
+    const int block = own ? p->block : 128, bps = own ? p->bps : 4, fs = own ? p->frame_smem : 0;
+    const long long tiles = (count + block - 1) / block;
+    const int grid = (int)std::min<long long>(tiles, (long long)p->sm_count * bps);
+    st = ensure_frame(p, grid, block, frame_units(p));
     if (st) return st;
-    KParams K = make_params(p, p->frame_smem);
+    KParams K = make_params(p, fs);
     K.frame_units = frame_units(p);
-    K.tile = p->block;
+    K.tile = block;
     K.outF = dF ? out_F : tF;
     K.outFc = out_Fc ? (dFc ? out_Fc : tFc) : nullptr;
     K.outG = out_G ? (dG ? out_G : tG) : nullptr;
     K.store_first_g = first;
-    CK(launch_bound(kernel_mode(p, true), K, grid, p->block, smem_bytes(p, p->block, p->frame_smem), s));
+    CK(launch_bound(kernel_mode(p, true), K, grid, block, smem_bytes(p, block, fs), s));
     p->launches += 1;
     if (!dF) CK(cudaMemcpyAsync(out_F, tF, fb, cudaMemcpyDeviceToHost, s));
     if (out_Fc && !dFc) CK(cudaMemcpyAsync(out_Fc, tFc, fb, cudaMemcpyDeviceToHost, s));
@@ -988,7 +998,7 @@ extern "C" ivb_status ivb_specialize_compile(const ivb_tape* tape, int32_t grad_
         ivb_options_default(&o);
         if (compact == 4) o.seg_ilp = 2;
         const SegPolicy pol = seg_policy(o);
-        const SegSource src = jit_seg_source(P, ins, rins, consts, kJitBlockMax, seg_min_blocks(pol.max_regs),
+        const SegSource src = jit_seg_source(P, ins, rins, consts, seg_block_max(pol.max_regs),
                                              compact == 4 ? 15 : kJitDefaultEmulate, 0, pol);
         e = jit_seg_compile(src, pol.max_regs, cubin, tables, seconds, &regs, &spill);
     } else {

@@ -74,6 +74,21 @@ struct Sub {
     const char* rec;     // the node's queue record
 };
 
+// Subdomains a block grabs at a time. With one pass per grab (tile == per) the
+// call's n subdomains are dealt out evenly: as many passes as full grabs would
+// take, each of the smallest whole number of warps that covers them, instead
+// of full passes and a last one that leaves most SMs idle. A pass of fewer
+// warps is shorter, since the warps of an SM share its pipes (1024-thread blocks,
+// configuration 5, 2^19 subdomains, 3.4 full passes: 62.8 -> 56.0 ms; configuration
+// 3, 941192 subdomains, 6.05 full passes: 8.6 -> 8.2 ms).
+__device__ __forceinline__ long long even_tile(long long n, int per, int tile) {
+    if (tile != per || n <= 0 || n >= (1LL << 31)) return tile;
+    const unsigned all = gridDim.x * (unsigned)per, m = (unsigned)n;
+    const unsigned passes = (m - 1u) / all + 1u;
+    const unsigned q = ((m - 1u) / (gridDim.x * passes) / 32u + 1u) * 32u;
+    return q < (unsigned)per ? (long long)q : tile;
+}
+
 // Blocks grab tiles of the global subdomain index space from a device counter
 // and map indices to nodes through the queue's prefix sums; body(sub) runs
 // for every lane of every pass (idle lanes included, for the warp reductions).
@@ -88,13 +103,14 @@ __device__ __forceinline__ void tile_loop_per(const KParams& P, const int per, B
     const long long* off = reinterpret_cast<const long long*>(P.queue + kQueueHeader);
     const char* recs = P.queue + kQueueHeader + 8 * (long long)(n_nodes + 1);
     __shared__ long long s_base;
+    const long long tile = even_tile(total - P.store_first_g, per, P.tile);
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) s_base = (long long)atomicAdd(P.counter, (unsigned long long)P.tile);
+        if (threadIdx.x == 0) s_base = (long long)atomicAdd(P.counter, (unsigned long long)tile);
         __syncthreads();
         const long long base = s_base;
         if (base >= total) break;
-        const long long end = base + P.tile < total ? base + P.tile : total;
+        const long long end = base + tile < total ? base + tile : total;
         for (long long g0 = base; g0 < end; g0 += per) {
             Sub s;
             s.g = g0 + (int)(threadIdx.x % (unsigned)per);

@@ -20,10 +20,17 @@ namespace ivb {
 
 // generated kernels: __launch_bounds__(kJitBlockMax, kJitMinBlocks), i.e. at
 // most 128 registers per thread; specialize = -1 compiles tapes of at most
-// kJitAutoMaxOps interval operations per subdomain (beyond that, compile time
-// grows to tens of seconds and the interpreter was within 5 % on the
-// configurations measured)
-constexpr int kJitBlockMax = 256, kJitMinBlocks = 2, kJitAutoMaxOps = 1024;
+// kJitAutoMaxOps interval operations per subdomain as one program (beyond that,
+// compile time grows to tens of seconds and the interpreter was within 5 % on
+// the configurations measured). In adjoint mode the segmented kernel takes
+// over from kSegMinOps on: with 32 warps per SM it is ahead at 620 operations
+// (configuration 2, 16 nodes x 16^4: 2.4 to 2.6 ms against 2.75) and compiles in a
+// tenth of the time; below, there is little to cut.
+constexpr int kJitBlockMax = 256, kJitMinBlocks = 2, kJitAutoMaxOps = 1024, kSegMinOps = 256;
+// chunks from which a segmented kernel keeps its warps on one chunk by default
+// (the autotuner times both): 306 chunks 56 ms with the barriers, 178 without;
+// 27 chunks 8.8 and 8.2 ms; 12 chunks 5.1 and 4.7 ms
+constexpr int kSegSyncChunks = 96;
 // endpoint operations emulated on the integer pipes by default (ivb_iv.cuh
 // policy bits): none -- on configuration 2 no policy beat the FP64 pipe alone
 // by more than the noise (the kernel runs at its 128-register cap with 16
@@ -63,9 +70,16 @@ struct SegPolicy {
     int chunk_stmts = 96;        // statements per chunk
     int recompute = 0;           // measured fastest: recomputation adds FP64 work, the state area streams with room to spare
     int units = 16;
-    int max_regs = 128;          // register budget of every chunk function
+    // register budget of every chunk function: 64 lets one block of 32 warps fill
+    // an SM (configuration 5, 2^19 subdomains: 72 registers and 28 warps 55 ms, 80
+    // and 24 60 ms, 128 and 16 67 ms; as two blocks of 8 warps, which stream
+    // through the code separately, 82 ms)
+    int max_regs = 64;
     int ilp = 1;                 // subdomains per thread (1, or 2 interleaved)
-    int outline = 1;             // short interval operations out of line: 0 none, 1 all, 2 products only
+    // short interval operations out of line: 0 none, 1 all, 2 products only (a
+    // call costs more than the two instructions of a sum: configuration 5 56 ms
+    // against 57 with 1, configuration 3 8.8 against 9.0, and 9.6 with 0)
+    int outline = 2;
 };
 struct SegSource {
     std::string kernel;               // tile loop, Step 1, chunk calls, Step 3 (one kernel per T)
@@ -76,8 +90,7 @@ struct SegSource {
     std::string error;                // "" unless the program could not be planned
 };
 SegSource jit_seg_source(const HostProgram& P, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
-                         const std::vector<double>& consts, int block_max, int min_blocks, int emulate, int form,
-                         const SegPolicy& pol);
+                         const std::vector<double>& consts, int block_max, int emulate, int form, const SegPolicy& pol);
 // compile the units in parallel and link them; "" on success
 std::string jit_seg_compile(const SegSource& src, int max_regs, std::vector<char>& cubin, std::string& tables_name,
                             double* seconds, int* registers, int* spill_bytes);

@@ -754,13 +754,13 @@ int slot_fc(int n, int o) { return 2 * n + 2 * o + 1; }
 // bound) are combined through shared memory by the objective's group; each
 // group reduces its own outputs' hulls. T = 1 is the plain kernel.
 std::string kernel_fn(const Builder& B, const Plan& pl, const std::vector<std::vector<int>>& groups, int T,
-                      bool sync, int K, int ns, const std::string& name, int block_max, int min_blocks) {
+                      bool sync, int K, int ns, const std::string& name, int block_max) {
     const int n = B.n, no = B.no, obj = B.P.obj;
     int gobj = 0;
     for (int g = 0; g < T; ++g)
         for (int o : groups[g]) if (o == obj) gobj = g;
     auto sub = [&](int k) { return "s" + S(k); };
-    std::string s = "extern \"C\" __global__ void __launch_bounds__(" + S(block_max) + ", " + S(min_blocks) + ") " +
+    std::string s = "extern \"C\" __global__ void __launch_bounds__(" + S(block_max) + ", 1) " +
                     name + "(const ivb::KParams P) {\n";
     s += "  using namespace ivb;\n";
     s += "  double* const st = P.gframe + (size_t)blockIdx.x * P.frame_units * blockDim.x + threadIdx.x;\n";
@@ -937,8 +937,7 @@ void compile_unit(const std::string& src, bool kernel, int max_regs, UnitResult&
 }  // namespace
 
 SegSource jit_seg_source(const HostProgram& P, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
-                         const std::vector<double>& consts, int block_max, int min_blocks, int emulate, int form,
-                         const SegPolicy& pol) {
+                         const std::vector<double>& consts, int block_max, int emulate, int form, const SegPolicy& pol) {
     Builder B{P, ins.data(), rins.data(), consts.data(), P.n_vars, P.n_out, form, form == 1};
     const int n = B.n, no = B.no;
     std::map<int, int> fixed;
@@ -991,8 +990,8 @@ SegSource jit_seg_source(const HostProgram& P, const std::vector<Ins>& ins, cons
         out.ts.push_back(T);
         const std::vector<std::vector<int>> groups = group_outputs(B, T);
         k += kernel_fn(B, pl, groups, T, false, K, ns, T == 1 ? "ivb_jit_bound" : "ivb_jit_bound_t" + S(T),
-                       block_max, min_blocks);
-        k += kernel_fn(B, pl, groups, T, true, K, ns, "ivb_jit_bound_t" + S(T) + "_sync", block_max, min_blocks);
+                       block_max);
+        k += kernel_fn(B, pl, groups, T, true, K, ns, "ivb_jit_bound_t" + S(T) + "_sync", block_max);
     }
     out.kernel = k;
     // chunks spread over units of similar size, compiled in parallel

@@ -27,7 +27,8 @@ struct KParams {
     const char* queue;     // device node queue (layout above)
     int32_t rec_bytes;
     unsigned long long* counter;   // work counter: first global index to hand out
-    int32_t tile;          // subdomains a block takes at a time (multiple of its subdomains per pass)
+    int32_t tile;          // subdomains a block takes at a time (multiple of its subdomains per pass; one
+                           // pass: at most that many, dealt out evenly)
     // per-thread frames (interpreter only)
     double* gframe;        // global frames: frame_units * blockDim per block
     int32_t frame_in_smem;
@@ -37,7 +38,7 @@ struct KParams {
     double* outF;          // store modes
     double* outFc;
     double* outG;
-    long long store_first_g;
+    long long store_first_g;   // first global index of the call (0 in the reduce modes)
     int32_t form;          // 0 MVF, 1 NIE, 2 MVF meet NIE
 };
 
