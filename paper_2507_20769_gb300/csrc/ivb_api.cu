@@ -239,11 +239,12 @@ std::vector<int> tpsub_choices(const ivb_problem* p) {
     return v;
 }
 
-// chunk synchronisation choices: the segmented kernels come with and without
+// chunk synchronisation choices: the segmented kernels come with and without;
+// programs larger than the instruction caches always keep their warps together
 std::vector<bool> sync_choices(const ivb_problem* p) {
     if (!reduce_jit(p) || !p->jit.kern_sync[0]) return {false};
     if (p->opt.seg_sync == 0) return {false};
-    if (p->opt.seg_sync == 1) return {true};
+    if (p->opt.seg_sync == 1 || p->jit.chunks >= kSegSyncChunks) return {true};
     return {false, true};
 }
 
@@ -382,8 +383,7 @@ ivb_status default_tuning(ivb_problem* p) {
     else p->frame_smem = (bytes + 1024 <= (size_t)p->smem_optin && bytes * p->bps <= 220 * 1024) ? 1 : 0;
     p->tpsub = tpsub_choices(p).front();
     if (p->block < 32 * p->tpsub) p->tpsub = 1;
-    // code larger than the instruction caches: keep the warps on one chunk
-    p->chunk_sync = seg && p->jit.chunks >= kSegSyncChunks ? sync_choices(p).back() : sync_choices(p).front();
+    p->chunk_sync = sync_choices(p).front();
     const int occ = reduce_occupancy(p, p->block, p->frame_smem, p->tpsub, p->chunk_sync);
     if (occ < 1) return fail(p, IVB_ENOTSUP, "launch configuration does not fit on an SM");
     if (p->bps > occ) p->bps = occ;

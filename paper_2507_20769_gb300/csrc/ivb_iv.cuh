@@ -242,6 +242,48 @@ __device__ __forceinline__ iv iv_fma(iv x, iv y, iv acc) {
     return mk(lo, hi);
 }
 
+// products by a nonzero constant, for the generated kernels: the sign is known,
+// so there is nothing to select; x * 2^K is an exponent step without FP64
+// (more than half of the constant factors of the workload tapes are powers of
+// two). The results are the bits of iv_mul and iv_fma with [c, c].
+__device__ __forceinline__ iv iv_mulc(iv x, double c) {
+    const double a = c > 0.0 ? x.lo : x.hi, b = c > 0.0 ? x.hi : x.lo;
+    double lo = __dmul_rd(a, c), hi = __dmul_ru(b, c);
+    if (__any_sync(__activemask(), odd_product(lo) | odd_product(hi))) {
+        if (is0(a)) lo = 0.0;
+        if (is0(b)) hi = 0.0;
+    }
+    return mk(lo, hi);
+}
+template <int K, bool NEG> __device__ __forceinline__ double scaled(double x) {
+    return from_bits((bits(x) + K * (1LL << 52)) ^ (NEG ? (long long)0x8000000000000000ULL : 0LL));
+}
+// exponent field outside [A, B]
+template <int A, int B> __device__ __forceinline__ bool exponent_outside(double x) {
+    return 2u * (unsigned)((unsigned long long)bits(x) >> 32) - ((unsigned)A << 21) >= ((unsigned)(B - A + 1) << 21);
+}
+template <int K, bool NEG> __device__ __forceinline__ iv iv_mul_pow2(iv x, double c) {   // c = +-2^K, |K| <= 1000
+    const double a = NEG ? x.hi : x.lo, b = NEG ? x.lo : x.hi;
+    double lo = scaled<K, NEG>(a), hi = scaled<K, NEG>(b);
+    constexpr int A = K < 0 ? 1 - K : 1, B = K > 0 ? 2046 - K : 2046;
+    if (__any_sync(__activemask(), exponent_outside<A, B>(a) | exponent_outside<A, B>(b))) {
+        lo = is0(a) ? 0.0 : __dmul_rd(a, c);
+        hi = is0(b) ? 0.0 : __dmul_ru(b, c);
+    }
+    return mk(lo, hi);
+}
+__device__ __forceinline__ iv iv_fmac(iv x, double c, iv acc) {
+    const double a = c > 0.0 ? x.lo : x.hi, b = c > 0.0 ? x.hi : x.lo;
+    double lo = __fma_rd(a, c, acc.lo), hi = __fma_ru(b, c, acc.hi);
+    if (__any_sync(__activemask(), odd_product(lo) | odd_product(hi))) {
+        if (is0(a)) lo = acc.lo;
+        if (is0(b)) hi = is0(acc.hi) ? 0.0 : acc.hi;
+    }
+    return mk(lo, hi);
+}
+// [0,0] + x
+__device__ __forceinline__ iv iv_from_zero(iv x) { return mk(x.lo, is0(x.hi) ? 0.0 : x.hi); }
+
 // 2*x rounded toward -inf / +inf: exact (an exponent increment on the integer
 // pipe, or a shift for zero and subnormals) unless |x| >= 2^1023, where the
 // directed multiply decides between the largest double and infinity

@@ -27,10 +27,12 @@ namespace ivb {
 // (configuration 2, 16 nodes x 16^4: 2.4 to 2.6 ms against 2.75) and compiles in a
 // tenth of the time; below, there is little to cut.
 constexpr int kJitBlockMax = 256, kJitMinBlocks = 2, kJitAutoMaxOps = 1024, kSegMinOps = 256;
-// chunks from which a segmented kernel keeps its warps on one chunk by default
-// (the autotuner times both): 306 chunks 56 ms with the barriers, 178 without;
-// 27 chunks 8.8 and 8.2 ms; 12 chunks 5.1 and 4.7 ms
-constexpr int kSegSyncChunks = 96;
+// chunks from which a segmented kernel keeps its warps on one chunk (below, the
+// autotuner times both). Warps that drift apart stream through the code
+// separately, and a sample of uniform subdomains does not show it: 306 chunks 56
+// ms with the barriers, 178 without; 27 chunks 8.8 and 8.2 ms on one uniform batch
+// (configuration 3), but 37 and 45 ms on 256 uneven nodes; 12 chunks 4.4 and 4.0 ms
+constexpr int kSegSyncChunks = 20;
 // endpoint operations emulated on the integer pipes by default (ivb_iv.cuh
 // policy bits): none -- on configuration 2 no policy beat the FP64 pipe alone
 // by more than the noise (the kernel runs at its 128-register cap with 16

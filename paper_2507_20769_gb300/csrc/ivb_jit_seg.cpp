@@ -13,9 +13,10 @@
 // cut into short chunks, each a function of its own, with a bound on the
 // estimated work and on the values each chunk keeps in registers:
 //  * a value that crosses a chunk boundary lives in a per-thread state area
-//    in global memory (element u of thread t at state[u * blockDim + t],
-//    coalesced across a warp), stored right after the statement that writes
-//    it and loaded where the next chunk first reads it;
+//    in global memory (element u of lane l at state[u * 32 + l] of its warp's
+//    area: coalesced, and a constant offset from one pointer), stored right
+//    after the statement that writes it and loaded where the next chunk first
+//    reads it;
 //  * with a recomputation policy a reverse chunk does not read the forward
 //    values of its own segment from memory: it recomputes them from the
 //    segment's checkpoints (the values that enter the segment from earlier
@@ -41,6 +42,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -107,6 +109,7 @@ struct Builder {
     std::vector<std::string> vname;
     std::vector<int> vtype;
     std::map<std::string, int> vid;
+    std::vector<bool> g_zero;   // G_i of the output being written: no contribution yet
 
     int var(const std::string& nm, int type = V_IV) {
         auto it = vid.find(nm);
@@ -139,6 +142,19 @@ struct Builder {
         return konst(idx);
     }
 
+    // x * [c, c] and acc + x * [c, c]: 14 % of the FP64 instructions of
+    // configuration 5 were products by powers of two (with the per-warp state
+    // area: 152 -> 134 ms on 6 x 2^18 subdomains; configuration 2 9.07 -> 8.25 ms)
+    static std::string mul_const(const std::string& x, double c) {
+        int e = 0;
+        if (std::fabs(std::frexp(c, &e)) == 0.5 && e - 1 >= -1000 && e - 1 <= 1000)
+            return "iv_mul_pow2<" + S(e - 1) + (c < 0 ? ", true>(" : ", false>(") + x + ", " + lit(c) + ")";
+        return "iv_mulc(" + x + ", " + lit(c) + ")";
+    }
+    static std::string fma_const(const std::string& x, double c, const std::string& acc) {
+        return "iv_fmac(" + x + ", " + lit(c) + ", " + acc + ")";
+    }
+
     static std::string eval(uint32_t op, const std::string& A, const std::string& B) {
         switch (op) {
         case OP_ADD: return "iv_add(" + A + ", " + B + ")";
@@ -161,7 +177,10 @@ struct Builder {
         const std::string B = bk != K_NONE ? val(role, bk, I.w1 >> 16, s.reads) : A;
         const std::string D = std::string(1, role) + S(dst);
         s.writes.push_back(var(D));
-        s.code = D + "$ = " + eval(op, A, B) + ";";
+        // a constant factor (commuted products have the same bits)
+        const double ca = ak == K_CONST ? consts[I.w1 & 0xFFFFu] : 0.0, cb = bk == K_CONST ? consts[I.w1 >> 16] : 0.0;
+        const bool kc = op == OP_MUL && (cb != 0.0 || ca != 0.0);
+        s.code = D + "$ = " + (kc ? (cb != 0.0 ? mul_const(A, cb) : mul_const(B, ca)) : eval(op, A, B)) + ";";
         s.cost = op_cost(op);
         s.op = op;
         s.phase = role == 'r' ? 1 : 0;
@@ -178,8 +197,13 @@ struct Builder {
         s.reads.push_back(var("w" + S(wslot)));
         if (op == OP_VAR) {
             const std::string g = "g" + S(R.w1);
-            s.reads.push_back(var(g));
             s.writes.push_back(var(g));
+            if (g_zero[R.w1]) {   // the first contribution to G_i
+                g_zero[R.w1] = false;
+                s.code = g + "$ = iv_from_zero(" + W + ");";
+                return s;
+            }
+            s.reads.push_back(var(g));
             s.code = g + "$ = iv_add(" + g + "$, " + W + ");";
             s.cost = 2.0;
             return s;
@@ -192,6 +216,7 @@ struct Builder {
         auto V = [&]() { return rv(K_SLOT, R.w3 & 0xFFFFu); };
         std::string ax = "W", ay, bx = "W", by;
         bool a_prod = true, b_prod = true, sub_a = false, sub_b = false;
+        double a_const = 0.0, b_const = 0.0;   // nonzero: the second factor of the contribution
         std::string body = "const auto W = " + W + "; ";
         double cost = 0.0;
         switch (op) {
@@ -201,6 +226,8 @@ struct Builder {
         case OP_MUL:
             if (!a_none) ay = rv(Bk, R.w2 >> 16);
             if (!b_none) by = rv(Ak, R.w2 & 0xFFFFu);
+            if (Bk == K_CONST) a_const = consts[R.w2 >> 16];
+            if (Ak == K_CONST) b_const = consts[R.w2 & 0xFFFFu];
             break;
         case OP_DIV:
             body += "const auto Rb = iv_recip(" + rv(Bk, R.w2 >> 16) + "); ";
@@ -219,13 +246,14 @@ struct Builder {
         case OP_LOG: if (!a_none) { ay = "iv_recip_pos(" + rv(Ak, R.w2 & 0xFFFFu) + ")"; cost += 4.0; } break;
         default: a_prod = b_prod = false; ax = bx = "entire()";
         }
-        if (!a_none && a_prod) body += "const auto ya = " + ay + "; ";
-        if (!b_none && b_prod) body += "const auto yb = " + by + "; ";
+        if (!a_none && a_prod && a_const == 0.0) body += "const auto ya = " + ay + "; ";
+        if (!b_none && b_prod && b_const == 0.0) body += "const auto yb = " + by + "; ";
         std::string upd;
         if (!a_none) {
             const std::string un = "w" + S(R.w1 & 0xFFFFu), u = un + "$";
             std::string v;
-            if (a_prod) v = a_init ? "iv_mul(" + ax + ", ya)" : "iv_fma(" + ax + ", ya, " + u + ")";
+            if (a_prod && a_const != 0.0) v = a_init ? mul_const(ax, a_const) : fma_const(ax, a_const, u);
+            else if (a_prod) v = a_init ? "iv_mul(" + ax + ", ya)" : "iv_fma(" + ax + ", ya, " + u + ")";
             else if (a_init) v = sub_a ? "iv_neg(" + ax + ")" : ax;
             else v = sub_a ? "iv_sub(" + u + ", " + ax + ")" : "iv_add(" + u + ", " + ax + ")";
             if (!a_init) s.reads.push_back(var(un));
@@ -235,7 +263,8 @@ struct Builder {
         if (!b_none) {
             const std::string un = "w" + S(R.w1 >> 16), u = un + "$";
             std::string v;
-            if (b_prod) v = b_init ? "iv_mul(" + bx + ", yb)" : "iv_fma(" + bx + ", yb, " + u + ")";
+            if (b_prod && b_const != 0.0) v = b_init ? mul_const(bx, b_const) : fma_const(bx, b_const, u);
+            else if (b_prod) v = b_init ? "iv_mul(" + bx + ", yb)" : "iv_fma(" + bx + ", yb, " + u + ")";
             else if (b_init) v = sub_b ? "iv_neg(" + bx + ")" : bx;
             else v = sub_b ? "iv_sub(" + u + ", " + bx + ")" : "iv_add(" + u + ", " + bx + ")";
             if (!b_init) s.reads.push_back(var(un));
@@ -311,10 +340,15 @@ struct Builder {
                 Stmt t;
                 t.out = o;
                 t.phase = 2;
-                for (int i = 0; i < n; ++i) {
-                    t.writes.push_back(var("g" + S(i)));
-                    t.code += "g" + S(i) + "$ = zero(); ";
-                }
+                g_zero.assign(n, true);
+                std::vector<bool> reached(n, false);
+                for (int i = A.rv_begin; i < A.rv_begin + A.rv_count; ++i)
+                    if ((rins[i].w0 & 31u) == OP_VAR) reached[rins[i].w1] = true;
+                for (int i = 0; i < n; ++i)
+                    if (!reached[i]) {
+                        t.writes.push_back(var("g" + S(i)));
+                        t.code += "g" + S(i) + "$ = zero(); ";
+                    }
                 if (A.out_wslot >= 0) {
                     t.writes.push_back(var("w" + S(A.out_wslot)));
                     t.code += "w" + S(A.out_wslot) + "$ = one();";
@@ -339,9 +373,8 @@ struct Builder {
                 m.code = "{ auto mvf = fc" + S(o) + "$; ";
                 for (int i = 0; i < n; ++i) {
                     m.reads.push_back(var("g" + S(i)));
-                    m.reads.push_back(var("X" + S(i)));
-                    m.reads.push_back(var("c" + S(i), V_DBL));
-                    m.code += "mvf = mvf_term(mvf, g" + S(i) + "$, X" + S(i) + "$, c" + S(i) + "$); ";
+                    m.reads.push_back(var("D" + S(i)));
+                    m.code += "mvf = iv_fma(g" + S(i) + "$, D" + S(i) + "$, mvf); ";   // mvf_term
                 }
                 m.reads.push_back(var("nie" + S(o)));
                 m.code += F + "$ = final_form(" + S(form) + ", mvf, nie" + S(o) + "$); }";
@@ -458,7 +491,7 @@ std::vector<Chunk> cut(const Builder& B, const std::vector<Stmt>& prog, double b
 }
 
 // Liveness over one program's chunks and state slots for the values that
-// cross chunk boundaries. Variables with a fixed slot (X_i, c_i, f(c)_o, F_o)
+// cross chunk boundaries. Variables with a fixed slot (X_i, c_i, X_i - c_i, f(c)_o, F_o)
 // always live there; the others take working slots from `w0` on, released
 // one chunk after their last read (inside a chunk a live-in may be loaded
 // after another variable's store).
@@ -579,14 +612,14 @@ const char* kPair =
     "};\n"
     "struct d2 { double a, b; };\n"
     "__device__ __forceinline__ iv2 mk(d2 x, d2 y) { return iv2(mk(x.a, y.a), mk(x.b, y.b)); }\n"
-    "__device__ __forceinline__ iv2 ld2(const double* st, int ss, int slot, int ns) {\n"
-    "  return iv2(st_ld(st, ss, slot), st_ld(st, ss, slot + ns)); }\n"
-    "__device__ __forceinline__ d2 ldd2(const double* st, int ss, int slot, int ns) {\n"
-    "  d2 r; r.a = st_d(st, ss, slot); r.b = st_d(st, ss, slot + ns); return r; }\n"
-    "__device__ __forceinline__ void st2(double* st, int ss, int slot, int ns, const iv2& v) {\n"
-    "  st_st(st, ss, slot, v.a); st_st(st, ss, slot + ns, v.b); }\n"
-    "__device__ __forceinline__ void std2(double* st, int ss, int slot, int ns, const d2& v) {\n"
-    "  st_sd(st, ss, slot, v.a); st_sd(st, ss, slot + ns, v.b); }\n"
+    "__device__ __forceinline__ iv2 ld2(const double* st, int slot, int ns) {\n"
+    "  return iv2(st_ld(st, slot), st_ld(st, slot + ns)); }\n"
+    "__device__ __forceinline__ d2 ldd2(const double* st, int slot, int ns) {\n"
+    "  d2 r; r.a = st_d(st, slot); r.b = st_d(st, slot + ns); return r; }\n"
+    "__device__ __forceinline__ void st2(double* st, int slot, int ns, const iv2& v) {\n"
+    "  st_st(st, slot, v.a); st_st(st, slot + ns, v.b); }\n"
+    "__device__ __forceinline__ void std2(double* st, int slot, int ns, const d2& v) {\n"
+    "  st_sd(st, slot, v.a); st_sd(st, slot + ns, v.b); }\n"
     "static __device__ __noinline__ iv2 o_add(iv2 x, iv2 y) {\n"
     "  return iv2(iv_add_t<0>(x.a, y.a), iv_add_t<IVB_EMU_B>(x.b, y.b)); }\n"
     "static __device__ __noinline__ iv2 o_sub(iv2 x, iv2 y) {\n"
@@ -604,8 +637,12 @@ const char* kPair =
     "static __device__ __noinline__ iv2 iv_recip_pos(iv2 x) { return iv2(iv_recip_pos(x.a), iv_recip_pos(x.b)); }\n"
     "__device__ __forceinline__ iv2 iv_neg(iv2 x) { return iv2(iv_neg(x.a), iv_neg(x.b)); }\n"
     "__device__ __forceinline__ iv2 iv_twice(iv2 x) { return iv2(iv_twice(x.a), iv_twice(x.b)); }\n"
-    "__device__ __forceinline__ iv2 mvf_term(iv2 acc, iv2 g, iv2 x, d2 c) {\n"
-    "  return iv2(mvf_term(acc.a, g.a, x.a, c.a), mvf_term(acc.b, g.b, x.b, c.b)); }\n"
+    "__device__ __forceinline__ iv2 iv_mulc(iv2 x, double c) { return iv2(iv_mulc(x.a, c), iv_mulc(x.b, c)); }\n"
+    "template <int K, bool NEG> __device__ __forceinline__ iv2 iv_mul_pow2(iv2 x, double c) {\n"
+    "  return iv2(iv_mul_pow2<K, NEG>(x.a, c), iv_mul_pow2<K, NEG>(x.b, c)); }\n"
+    "__device__ __forceinline__ iv2 iv_fmac(iv2 x, double c, iv2 z) {\n"
+    "  return iv2(iv_fmac(x.a, c, z.a), iv_fmac(x.b, c, z.b)); }\n"
+    "__device__ __forceinline__ iv2 iv_from_zero(iv2 x) { return iv2(iv_from_zero(x.a), iv_from_zero(x.b)); }\n"
     "__device__ __forceinline__ iv2 final_form(int f, iv2 m, iv2 v) {\n"
     "  return iv2(final_form(f, m.a, v.a), final_form(f, m.b, v.b)); }\n"
     "}\n";
@@ -617,7 +654,7 @@ std::string chunk_fn_pair(const Builder& B, const Plan& pl, int c, int ns) {
     const std::map<int, int>& stv = pl.store_slot[c];
     const std::string NS = S(ns);
     std::string s = "extern \"C\" __device__ __noinline__ void ivb_ck" + S(c) +
-                    "(double* __restrict__ st, const int ss) {\n  using namespace ivb;\n";
+                    "(double* __restrict__ st) {\n  using namespace ivb;\n";
     std::set<int> touched;
     for (const Stmt& t : ch.body) {
         for (int v : t.reads) touched.insert(v);
@@ -640,7 +677,7 @@ std::string chunk_fn_pair(const Builder& B, const Plan& pl, int c, int ns) {
         const Stmt& t = ch.body[i];
         for (int v : t.reads)
             if (!written.count(v) && !loaded.count(v)) {
-                s += "  " + B.vname[v] + (B.vtype[v] == V_DBL ? " = ldd2(st, ss, " : " = ld2(st, ss, ") +
+                s += "  " + B.vname[v] + (B.vtype[v] == V_DBL ? " = ldd2(st, " : " = ld2(st, ") +
                      S(ld.at(v)) + ", " + NS + ");\n";
                 loaded.insert(v);
             }
@@ -649,7 +686,7 @@ std::string chunk_fn_pair(const Builder& B, const Plan& pl, int c, int ns) {
         for (int v : t.writes) {
             auto it = stv.find(v);
             if (last_write[v] == i && it != stv.end())
-                s += std::string(B.vtype[v] == V_DBL ? "  std2(st, ss, " : "  st2(st, ss, ") + S(it->second) + ", " +
+                s += std::string(B.vtype[v] == V_DBL ? "  std2(st, " : "  st2(st, ") + S(it->second) + ", " +
                      NS + ", " + B.vname[v] + ");\n";
         }
     }
@@ -665,7 +702,7 @@ std::string chunk_fn(const Builder& B, const Plan& pl, int c, int K, int ns, int
     const std::map<int, int>& ld = pl.load_slot[c];
     const std::map<int, int>& stv = pl.store_slot[c];
     std::string s = "extern \"C\" __device__ __noinline__ void ivb_ck" + S(c) +
-                    "(double* __restrict__ st, const int ss) {\n  using namespace ivb;\n";
+                    "(double* __restrict__ st) {\n  using namespace ivb;\n";
     std::set<int> touched;
     for (const Stmt& t : ch.body) {
         for (int v : t.reads) touched.insert(v);
@@ -693,7 +730,7 @@ std::string chunk_fn(const Builder& B, const Plan& pl, int c, int K, int ns, int
             if (!written.count(v) && !loaded.count(v)) {
                 for (int k = 0; k < K; ++k) {
                     const int slot = ld.at(v) + k * ns;
-                    s += "  " + nm(v, k) + (B.vtype[v] == V_DBL ? " = st_d(st, ss, " : " = st_ld(st, ss, ") + S(slot) +
+                    s += "  " + nm(v, k) + (B.vtype[v] == V_DBL ? " = st_d(st, " : " = st_ld(st, ") + S(slot) +
                          ");\n";
                 }
                 loaded.insert(v);
@@ -704,7 +741,7 @@ std::string chunk_fn(const Builder& B, const Plan& pl, int c, int K, int ns, int
             auto it = stv.find(v);
             if (last_write[v] == i && it != stv.end())
                 for (int k = 0; k < K; ++k)
-                    s += std::string(B.vtype[v] == V_DBL ? "  st_sd(st, ss, " : "  st_st(st, ss, ") +
+                    s += std::string(B.vtype[v] == V_DBL ? "  st_sd(st, " : "  st_st(st, ") +
                          S(it->second + k * ns) + ", " + nm(v, k) + ");\n";
         }
     }
@@ -720,12 +757,11 @@ const char* kPrelude =
 
 const char* kStateHelpers =
     "namespace ivb {\n"
-    "__device__ __forceinline__ iv st_ld(const double* st, int ss, int slot) {\n"
-    "  return mk(st[(size_t)(2 * slot) * ss], st[(size_t)(2 * slot + 1) * ss]); }\n"
-    "__device__ __forceinline__ double st_d(const double* st, int ss, int slot) { return st[(size_t)(2 * slot) * ss]; }\n"
-    "__device__ __forceinline__ void st_st(double* st, int ss, int slot, iv v) {\n"
-    "  st[(size_t)(2 * slot) * ss] = v.lo; st[(size_t)(2 * slot + 1) * ss] = v.hi; }\n"
-    "__device__ __forceinline__ void st_sd(double* st, int ss, int slot, double v) { st[(size_t)(2 * slot) * ss] = v; }\n"
+    "__device__ __forceinline__ iv st_ld(const double* st, int slot) { return mk(st[64 * slot], st[64 * slot + 32]); }\n"
+    "__device__ __forceinline__ double st_d(const double* st, int slot) { return st[64 * slot]; }\n"
+    "__device__ __forceinline__ void st_st(double* st, int slot, iv v) {\n"
+    "  st[64 * slot] = v.lo; st[64 * slot + 32] = v.hi; }\n"
+    "__device__ __forceinline__ void st_sd(double* st, int slot, double v) { st[64 * slot] = v; }\n"
     "}\n";
 
 std::string unit_head(int emulate, bool kernel_unit, bool paired = false) {
@@ -740,11 +776,12 @@ std::string unit_head(int emulate, bool kernel_unit, bool paired = false) {
     return s;
 }
 
-// fixed state slots: X_i at i, c_i at n + i, F_o at 2n + 2o, f(c)_o at 2n + 2o + 1
+// fixed state slots: X_i at i, c_i at n + i, X_i - c_i at 2n + i, F_o at 3n + 2o, f(c)_o at 3n + 2o + 1
 int slot_X(int n, int i) { return i; }
 int slot_c(int n, int i) { return n + i; }
-int slot_F(int n, int o) { return 2 * n + 2 * o; }
-int slot_fc(int n, int o) { return 2 * n + 2 * o + 1; }
+int slot_D(int n, int i) { return 2 * n + i; }
+int slot_F(int n, int o) { return 3 * n + 2 * o; }
+int slot_fc(int n, int o) { return 3 * n + 2 * o + 1; }
 
 // One kernel per number T of threads sharing a subdomain: a block's threads
 // form T groups of blockDim/T (whole warps); group g runs the programs of its
@@ -763,8 +800,8 @@ std::string kernel_fn(const Builder& B, const Plan& pl, const std::vector<std::v
     std::string s = "extern \"C\" __global__ void __launch_bounds__(" + S(block_max) + ", 1) " +
                     name + "(const ivb::KParams P) {\n";
     s += "  using namespace ivb;\n";
-    s += "  double* const st = P.gframe + (size_t)blockIdx.x * P.frame_units * blockDim.x + threadIdx.x;\n";
-    s += "  const int ss = blockDim.x;\n";
+    s += "  double* const st = P.gframe + ((size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32) * P.frame_units * 32 +\n"
+         "                     threadIdx.x % 32;\n";
     s += "  const int per = blockDim.x / " + S(T) + ";\n";
     s += "  const int grp = threadIdx.x / per;\n";
     if (T > 1) s += "  __shared__ unsigned char s_fl[" + S(K) + "][" + S(block_max) + "];\n";
@@ -785,8 +822,9 @@ std::string kernel_fn(const Builder& B, const Plan& pl, const std::vector<std::v
         const std::string sk = k == 0 ? "s0" : "(s1.valid ? s1 : s0)";
         s += "      { const Sub& d = " + sk + "; unsigned int kk = d.k;\n";
         for (int i = 0; i < n; ++i)
-            s += "        { iv X; double c; decode_dim(d.rec, " + S(n) + ", " + S(i) + ", kk, X, c); st_st(st, ss, " +
-                 S(slot_X(n, i) + k * ns) + ", X); st_sd(st, ss, " + S(slot_c(n, i) + k * ns) + ", c); }\n";
+            s += "        { iv X; double c; decode_dim(d.rec, " + S(n) + ", " + S(i) + ", kk, X, c); st_st(st, " +
+                 S(slot_X(n, i) + k * ns) + ", X); st_sd(st, " + S(slot_c(n, i) + k * ns) + ", c);" +
+                 (B.nie_only ? "" : " st_st(st, " + S(slot_D(n, i) + k * ns) + ", off_centre(X, c));") + " }\n";
         s += "      }\n";
     }
     // with `sync`, the threads of a group wait for each other after every
@@ -797,9 +835,9 @@ std::string kernel_fn(const Builder& B, const Plan& pl, const std::vector<std::v
         std::string r;
         for (int c = pl.prog_first[prog]; c < pl.prog_first[prog] + pl.prog_count[prog]; ++c) {
             if (sync)
-                r += ind + "if (s0.valid) ivb_ck" + S(c) + "(st, ss);\n" + ind + "asm volatile(\"bar.sync " + S(1 + g) +
+                r += ind + "if (s0.valid) ivb_ck" + S(c) + "(st);\n" + ind + "asm volatile(\"bar.sync " + S(1 + g) +
                      ", %0;\" :: \"r\"(per) : \"memory\");\n";
-            else r += ind + "ivb_ck" + S(c) + "(st, ss);\n";
+            else r += ind + "ivb_ck" + S(c) + "(st);\n";
         }
         return r;
     };
@@ -814,13 +852,13 @@ std::string kernel_fn(const Builder& B, const Plan& pl, const std::vector<std::v
             s += ind + "  " + (sync ? "if (s0.valid) " : "") + "{\n";
             for (int k = 0; k < K; ++k) {
                 const std::string Fk = "F" + S(o) + "_" + S(k), fl = "fl_" + S(k);
-                s += ind + "    " + Fk + " = st_ld(st, ss, " + S(slot_F(n, o) + k * ns) + ");\n";
+                s += ind + "    " + Fk + " = st_ld(st, " + S(slot_F(n, o) + k * ns) + ");\n";
                 s += ind + "    if (excludes_feasible(" + S(B.P.out_kind[o]) + "u, " + Fk + ")) " + fl + " |= 1u;\n";
                 if (B.P.out_kind[o] == OUT_INEQ)
-                    s += ind + "    if (!le0(st_ld(st, ss, " + S(slot_fc(n, o) + k * ns) + ").hi)) " + fl + " |= 2u;\n";
+                    s += ind + "    if (!le0(st_ld(st, " + S(slot_fc(n, o) + k * ns) + ").hi)) " + fl + " |= 2u;\n";
                 if (o == obj) {
                     s += ind + "    obj_lo_" + S(k) + " = " + Fk + ".lo;\n";
-                    s += ind + "    fco_" + S(k) + " = st_ld(st, ss, " + S(slot_fc(n, o) + k * ns) + ").hi;\n";
+                    s += ind + "    fco_" + S(k) + " = st_ld(st, " + S(slot_fc(n, o) + k * ns) + ").hi;\n";
                 }
             }
             s += ind + "  }\n";
@@ -944,6 +982,7 @@ SegSource jit_seg_source(const HostProgram& P, const std::vector<Ins>& ins, cons
     for (int i = 0; i < n; ++i) {
         fixed[B.var("X" + S(i))] = slot_X(n, i);
         fixed[B.var("c" + S(i), V_DBL)] = slot_c(n, i);
+        fixed[B.var("D" + S(i))] = slot_D(n, i);
     }
     for (int o = 0; o < no; ++o) {
         fixed[B.var("F" + S(o))] = slot_F(n, o);
@@ -951,7 +990,7 @@ SegSource jit_seg_source(const HostProgram& P, const std::vector<Ins>& ins, cons
     }
     B.build();
     Plan pl;
-    pl.n_slots = 2 * n + 2 * no;
+    pl.n_slots = 3 * n + 2 * no;
     SegSource out;
     for (const Builder::Prog& pr : B.progs) {
         long long rec = 0;
@@ -967,7 +1006,7 @@ SegSource jit_seg_source(const HostProgram& P, const std::vector<Ins>& ins, cons
         }
         pl.prog_first.push_back((int)pl.chunks.size());
         pl.prog_count.push_back((int)ch.size());
-        const std::string e = plan_prog(B, ch, fixed, ends, 2 * n + 2 * no, pl);
+        const std::string e = plan_prog(B, ch, fixed, ends, 3 * n + 2 * no, pl);
         if (!e.empty()) { out.error = e; return out; }
         pl.chunks.insert(pl.chunks.end(), ch.begin(), ch.end());
         pl.recomputed += rec;
@@ -984,7 +1023,7 @@ SegSource jit_seg_source(const HostProgram& P, const std::vector<Ins>& ins, cons
     // programs of their own and there are at least T of them
     std::string k = unit_head(emulate, true);
     for (size_t c = 0; c < pl.chunks.size(); ++c)
-        k += "extern \"C\" __device__ void ivb_ck" + S(c) + "(double* __restrict__ st, const int ss);\n";
+        k += "extern \"C\" __device__ void ivb_ck" + S(c) + "(double* __restrict__ st);\n";
     for (int T : {1, 2, 4}) {
         if (T > 1 && (B.shared_point || no < T || block_max < 32 * T)) continue;
         out.ts.push_back(T);
