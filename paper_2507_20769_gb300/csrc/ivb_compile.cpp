@@ -343,4 +343,62 @@ std::string compile_tape(const ivb_tape* t, HostProgram& P, std::vector<Ins>& in
     return "";
 }
 
+void interpreter_programs(const HostProgram& P, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
+                          std::vector<XIns>& xins, std::vector<XRIns>& xrins) {
+    const FrameLayout& L = P.L;
+    // the point and the tangent sweep share their instructions, not their places: tangents
+    // behind the rest, then the outputs' forward programs on [c,c]
+    const int tan0 = (int)ins.size(), cone0 = tan0 + P.tan_count;
+    xins.assign((size_t)cone0 + ins.size() + 1, XIns{});
+    xrins.assign(rins.size() + 1, XRIns{});
+    // operand word of a value reference: slots are records of `rec` units from `base` on
+    auto word = [&](uint32_t kind, uint32_t idx, int base, int rec, bool point) -> uint32_t {
+        if (kind == K_SLOT) return (uint32_t)(base + (int)idx * rec) * 32u;
+        if (kind == K_CONST) return idx | kOpConst | kOpPoint;
+        if (kind == K_VAR) return point ? (uint32_t)(L.c_base + (int)idx) * 32u | kOpPoint : (uint32_t)(L.x_base + 2 * (int)idx) * 32u;
+        return 0u;
+    };
+    auto values = [&](int begin, int count, int base, int rec, bool point, int to) {
+        uint32_t last = ~0u;
+        for (int i = begin; i < begin + count; ++i) {
+            const Ins& I = ins[i];
+            const uint32_t op = I.w0 & 31u, ak = (I.w0 >> 5) & 3u, bk = (I.w0 >> 7) & 3u, ai = I.w1 & 0xFFFFu, bi = I.w1 >> 16;
+            XIns& X = xins[to + i - begin];
+            X.w = op | (ak == K_CONST ? 1u << 5 : 0u) | (bk == K_CONST || bk == K_NONE ? 1u << 6 : 0u) |
+                  (ak == K_VAR ? 1u << 7 | (ai & 0xFFu) << 16 : 0u) | (bk == K_VAR ? 1u << 8 | (bi & 0xFFu) << 24 : 0u);
+            X.dst = word(K_SLOT, I.w0 >> 16, base, rec, point);
+            X.a = word(ak, ai, base, rec, point);
+            X.b = bk == K_NONE ? X.a : word(bk, bi, base, rec, point);
+            if (X.a == last) X.a |= kOpLast;
+            if (X.b == last) X.b |= kOpLast;
+            last = X.dst;
+        }
+    };
+    values(P.pt_begin, P.pt_count, L.phase_base, 2, true, P.pt_begin);
+    values(P.tan_begin, P.tan_count, L.phase_base, L.tan_rec, false, tan0);
+    for (int o = 0; o < P.n_out; ++o) {
+        const AdjProgram& A = P.adj[o];
+        const int gb = L.phase_base, ab = gb + 2 * L.n, tb = ab + 2 * A.adj_slots;
+        values(A.fw_begin, A.fw_count, tb, 2, false, A.fw_begin);
+        values(A.fw_begin, A.fw_count, tb, 2, true, cone0 + A.fw_begin);
+        uint32_t last = ~0u;
+        for (int i = A.rv_begin; i < A.rv_begin + A.rv_count; ++i) {
+            const RIns& R = rins[i];
+            XRIns& X = xrins[i];
+            auto slot = [&](uint32_t k) { return (uint32_t)(ab + 2 * (int)k) * 32u; };
+            X.w = R.w0 & 0x1FFu;
+            X.slot = slot(R.w0 >> 16);
+            if (X.slot == last) X.w |= kAdjLast;
+            if ((R.w0 & 31u) == OP_VAR) { X.a_adj = (uint32_t)(gb + 2 * (int)R.w1) * 32u; continue; }
+            X.a_adj = slot(R.w1 & 0xFFFFu);
+            X.b_adj = slot(R.w1 >> 16);
+            if (!((R.w0 >> 8) & 1u)) last = X.b_adj;
+            else if (!((R.w0 >> 7) & 1u)) last = X.a_adj;
+            X.A = word((R.w3 >> 16) & 3u, R.w2 & 0xFFFFu, tb, 2, false);
+            X.B = word((R.w3 >> 18) & 3u, R.w2 >> 16, tb, 2, false);
+            X.V = word(K_SLOT, R.w3 & 0xFFFFu, tb, 2, false);
+        }
+    }
+}
+
 }  // namespace ivb

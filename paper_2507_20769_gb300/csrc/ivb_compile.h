@@ -17,4 +17,11 @@ std::string validate_tape(const ivb_tape* t);
 std::string compile_tape(const ivb_tape* t, HostProgram& P, std::vector<Ins>& ins, std::vector<RIns>& rins,
                          std::vector<double>& consts);
 
+// the interpreter's form of the value and reverse programs, entry by entry beside
+// `ins` and `rins`, then that of the tangent program, then the value programs of
+// the outputs' cones on [c,c], entry by entry again (one unread entry more at the
+// end, for the prefetch)
+void interpreter_programs(const HostProgram& P, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
+                          std::vector<XIns>& xins, std::vector<XRIns>& xrins);
+
 }  // namespace ivb

@@ -44,6 +44,25 @@ struct RIns {
     uint32_t w0, w1, w2, w3;
 };
 
+// The interpreter's form of the same programs: operands resolved to places in
+// memory, so that it decodes nothing but the operation. An operand word names a
+// double: frame element (unit * 32, the frames are laid out per warp) or, with
+// kOpConst, constant; its upper end lies 32 doubles further, with kOpPoint it is
+// the same double ([c,c] of a variable, constants). kOpLast: the result of the
+// instruction before.
+constexpr uint32_t kOpConst = 0x80000000u, kOpPoint = 0x40000000u, kOpLast = 0x20000000u, kOpIndex = 0x1FFFFFFFu;
+struct alignas(16) XIns {
+    // w = op[0:5) | a const[5] | b const or none[6] | a variable[7] | b variable[8] | a index[16:24) | b index[24:32)
+    uint32_t w, dst, a, b;
+};
+constexpr uint32_t kAdjLast = 1u << 9;   // the result's adjoint is what the instruction before stored last
+struct alignas(16) XRIns {
+    uint32_t w;               // the flags of RIns::w0 (bits 0..8), kAdjLast
+    uint32_t slot;            // adjoint of the result
+    uint32_t a_adj, b_adj;    // adjoints of the operands (op VAR: a_adj = gradient entry)
+    uint32_t A, B, V, pad;    // values: operand words; V a frame element
+};
+
 constexpr uint32_t kNoSlot = 0xFFFFu;
 
 // one output's adjoint program inside the flat instruction arrays
@@ -63,7 +82,8 @@ struct AdjProgram {
 //   [2n, 3n)                c_i
 //   [3n, 3n + 2 n_out)      f(c) of every output (point sweep results)
 //   [phase_base, ...)       phase region (reused by each phase)
-// Element u of thread t sits at frame[u * stride + t].
+// Element u of lane l sits at frame[u * 32 + l] of its warp's frame: coalesced,
+// and no multiply by the block size in the addresses.
 struct FrameLayout {
     int32_t n, n_out;
     int32_t x_base, c_base, fc_base, phase_base;

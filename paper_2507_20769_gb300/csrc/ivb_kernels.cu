@@ -14,6 +14,9 @@
 #include <cstdint>
 #include <cstring>
 
+// the interpreter's warps are at different instructions: one copy of the long
+// primitives keeps its code inside the instruction caches
+#define IVB_HEAVY static __noinline__
 #include "ivb_bound_common.cuh"
 #include "ivb_internal.h"
 #include "ivb_iv.cuh"
@@ -22,28 +25,35 @@
 namespace ivb {
 
 // ------------------------------------------------------------------ frame
+// this lane's element 0 of its warp's frame (units 32 doubles apart)
 struct Frame {
-    double* p;  // this thread's element 0
-    int s;      // stride between consecutive units
-    __device__ __forceinline__ double ld(int u) const { return p[(size_t)u * s]; }
-    __device__ __forceinline__ void st(int u, double v) const { p[(size_t)u * s] = v; }
+    double* p;
+    __device__ __forceinline__ double ld(int u) const { return p[u * 32]; }
+    __device__ __forceinline__ void st(int u, double v) const { p[u * 32] = v; }
     __device__ __forceinline__ iv get(int u) const { return mk(ld(u), ld(u + 1)); }
     __device__ __forceinline__ void put(int u, iv v) const { st(u, v.lo); st(u + 1, v.hi); }
+    // by element (unit * 32)
+    __device__ __forceinline__ iv at(uint32_t e) const { return mk(p[e], p[e + 32]); }
+    __device__ __forceinline__ void to(uint32_t e, iv v) const { p[e] = v.lo; p[e + 32] = v.hi; }
 };
 
 struct SweepCtx {
     Frame F;
     const double* consts;
-    int x_base, c_base;
-    bool point;  // VAR operands read [c,c] instead of X
+    int x_base;
 };
 
+// operand word (XIns)
+__device__ __forceinline__ iv operand(const SweepCtx& C, uint32_t w) {
+    const double* q = (w & kOpConst) ? C.consts : C.F.p;
+    q += w & kOpIndex;
+    const double lo = *q;
+    return mk(lo, (w & kOpPoint) ? lo : q[32]);
+}
+// value reference of an output: record of `rec` units from `base` on, variable or constant
 __device__ __forceinline__ iv load_val(const SweepCtx& C, uint32_t kind, uint32_t idx, int base, int rec) {
     if (kind == K_SLOT) return C.F.get(base + (int)idx * rec);
-    if (kind == K_VAR) {
-        if (C.point) { double c = C.F.ld(C.c_base + (int)idx); return mk(c, c); }
-        return C.F.get(C.x_base + 2 * (int)idx);
-    }
+    if (kind == K_VAR) return C.F.get(C.x_base + 2 * (int)idx);
     const double k = __ldg(C.consts + idx);
     return mk(k, k);
 }
@@ -63,175 +73,162 @@ __device__ __forceinline__ iv eval_value(uint32_t op, iv A, iv B) {
     return entire();
 }
 
-// interval values of a straight-line program; records of 2 units at `base`
-__device__ void run_values(const Ins* __restrict__ ins, int count, const SweepCtx& C, int base) {
+// Interval values of a straight-line program. The interpreter is bound by the
+// instructions around the arithmetic, not by the FP64 pipe (57 % busy): operands
+// come resolved to addresses, the next instruction is fetched ahead, and a
+// result that the next instruction reads stays in registers (configuration 3:
+// 385 k -> 290 k instructions per warp of subdomains). Barriers that keep the
+// warps on one handler cost more than they saved (13.1 ms without, 13.2 with one
+// every 16 instructions, 15.7 with one each).
+__device__ __noinline__ void run_values(const XIns* __restrict__ ins, int count, const SweepCtx C) {
+    uint4 I = __ldg(reinterpret_cast<const uint4*>(ins));
+    iv V = zero();
     for (int i = 0; i < count; ++i) {
-        const Ins I = ins[i];
-        const uint32_t op = I.w0 & 31u, ak = (I.w0 >> 5) & 3u, bk = (I.w0 >> 7) & 3u, dst = I.w0 >> 16;
-        const iv A = load_val(C, ak, I.w1 & 0xFFFFu, base, 2);
-        const iv B = (bk != K_NONE) ? load_val(C, bk, I.w1 >> 16, base, 2) : A;
-        C.F.put(base + 2 * (int)dst, eval_value(op, A, B));
+        const uint4 next = __ldg(reinterpret_cast<const uint4*>(ins + i + 1));
+        const uint32_t op = I.x & 31u;
+        const iv A = (I.z & kOpLast) ? V : operand(C, I.z);
+        const iv B = op > OP_DIV ? A : (I.w & kOpLast) ? V : operand(C, I.w);
+        V = eval_value(op, A, B);
+        C.F.to(I.y, V);
+        I = next;
     }
-}
-
-// tangent of an operand in direction d
-__device__ __forceinline__ iv load_tan(const SweepCtx& C, uint32_t kind, uint32_t idx, int base, int rec, int d) {
-    if (kind == K_SLOT) return C.F.get(base + (int)idx * rec + 2 + 2 * d);
-    if (kind == K_VAR) return ((int)idx == d) ? one() : zero();
-    return zero();
 }
 
 // forward-mode sweep: value + n tangent intervals per record (Section 3.2).
 // Terms whose tangent is exactly zero (constant operands) are skipped: adding
 // [0,0] and multiplying by [0,0] are exact, so the values do not change.
-__device__ void run_tangents(const Ins* __restrict__ ins, int count, const SweepCtx& C, int base, int n) {
-    const int rec = 2 * (1 + n);
+__device__ void run_tangents(const XIns* __restrict__ ins, int count, const SweepCtx& C, int n) {
+    uint4 I = __ldg(reinterpret_cast<const uint4*>(ins));
     for (int i = 0; i < count; ++i) {
-        const Ins I = ins[i];
-        const uint32_t op = I.w0 & 31u, ak = (I.w0 >> 5) & 3u, bk = (I.w0 >> 7) & 3u, dst = I.w0 >> 16;
-        const uint32_t ai = I.w1 & 0xFFFFu, bi = I.w1 >> 16;
-        const iv A = load_val(C, ak, ai, base, rec);
-        const iv B = (bk != K_NONE) ? load_val(C, bk, bi, base, rec) : A;
+        const uint4 next = __ldg(reinterpret_cast<const uint4*>(ins + i + 1));
+        const uint32_t op = I.x & 31u;
+        const bool az = (I.x >> 5) & 1u, bz = (I.x >> 6) & 1u, avar = (I.x >> 7) & 1u, bvar = (I.x >> 8) & 1u;
+        const uint32_t ai = (I.x >> 16) & 0xFFu, bi = I.x >> 24;
+        const uint32_t ea = I.z & ~kOpLast, eb = I.w & ~kOpLast;
+        const iv A = operand(C, ea);
+        const iv B = op > OP_DIV ? A : operand(C, eb);
         const iv V = eval_value(op, A, B);
-        const int o = base + (int)dst * rec;
-        const bool az = (ak == K_CONST), bz = (bk == K_CONST || bk == K_NONE);
+        // tangents of the operands in direction d (a variable's: the unit vector; a constant's: zero)
+        auto ta = [&](int d) { return az ? zero() : avar ? ((int)ai == d ? one() : zero()) : C.F.at(ea + 64u + 64u * d); };
+        auto tb = [&](int d) { return bz ? zero() : bvar ? ((int)bi == d ? one() : zero()) : C.F.at(eb + 64u + 64u * d); };
+        const uint32_t o = I.y + 64u;
         switch (op) {
         case OP_ADD:
-            for (int d = 0; d < n; ++d) {
-                iv t = az ? load_tan(C, bk, bi, base, rec, d)
-                          : bz ? load_tan(C, ak, ai, base, rec, d)
-                               : iv_add(load_tan(C, ak, ai, base, rec, d), load_tan(C, bk, bi, base, rec, d));
-                C.F.put(o + 2 + 2 * d, t);
-            }
-            break;
         case OP_SUB:
             for (int d = 0; d < n; ++d) {
-                iv t = az ? iv_neg(load_tan(C, bk, bi, base, rec, d))
-                          : bz ? load_tan(C, ak, ai, base, rec, d)
-                               : iv_sub(load_tan(C, ak, ai, base, rec, d), load_tan(C, bk, bi, base, rec, d));
-                C.F.put(o + 2 + 2 * d, t);
+                iv t = tb(d);
+                if (op == OP_SUB) t = iv_neg(t);
+                if (!az) t = bz ? ta(d) : iv_add(ta(d), t);
+                C.F.to(o + 64u * d, t);
             }
             break;
         case OP_NEG:
-            for (int d = 0; d < n; ++d) C.F.put(o + 2 + 2 * d, iv_neg(load_tan(C, ak, ai, base, rec, d)));
+            for (int d = 0; d < n; ++d) C.F.to(o + 64u * d, iv_neg(ta(d)));
             break;
         case OP_MUL:
+            if (az | bz)
+                for (int d = 0; d < n; ++d) C.F.to(o + 64u * d, iv_mul(az ? A : B, az ? tb(d) : ta(d)));
+            else
+                for (int d = 0; d < n; ++d) C.F.to(o + 64u * d, iv_fma(A, tb(d), iv_mul(ta(d), B)));
+            break;
+        default: {
+            // one factor for every direction: quotient, sqr, sqrt, exp, log
+            iv R = op == OP_DIV ? B : op == OP_EXP ? V : op == OP_LOG ? A : iv_twice(op == OP_SQR ? A : V);
+            if (op != OP_EXP && op != OP_SQR) R = op == OP_DIV || gt0(R.lo) ? iv_recip(R) : entire();
+            const iv Vn = iv_neg(V);
             for (int d = 0; d < n; ++d) {
                 iv t;
-                if (az) t = iv_mul(A, load_tan(C, bk, bi, base, rec, d));
-                else if (bz) t = iv_mul(load_tan(C, ak, ai, base, rec, d), B);
-                else t = iv_fma(A, load_tan(C, bk, bi, base, rec, d), iv_mul(load_tan(C, ak, ai, base, rec, d), B));
-                C.F.put(o + 2 + 2 * d, t);
+                if (op != OP_DIV || bz) t = ta(d);
+                else t = az ? iv_neg(iv_mul(V, tb(d))) : iv_fma(Vn, tb(d), ta(d));
+                C.F.to(o + 64u * d, iv_mul(t, R));
             }
-            break;
-        case OP_DIV: {
-            const iv R = iv_recip(B);
-            for (int d = 0; d < n; ++d) {
-                iv t;
-                if (bz) t = iv_mul(load_tan(C, ak, ai, base, rec, d), R);
-                else if (az) t = iv_mul(iv_neg(iv_mul(V, load_tan(C, bk, bi, base, rec, d))), R);
-                else t = iv_mul(iv_fma(iv_neg(V), load_tan(C, bk, bi, base, rec, d), load_tan(C, ak, ai, base, rec, d)), R);
-                C.F.put(o + 2 + 2 * d, t);
-            }
-        } break;
-        case OP_SQR: {
-            const iv D = iv_twice(A);
-            for (int d = 0; d < n; ++d) C.F.put(o + 2 + 2 * d, iv_mul(D, load_tan(C, ak, ai, base, rec, d)));
-        } break;
-        case OP_SQRT: {
-            const iv R = iv_recip_pos(iv_twice(V));
-            for (int d = 0; d < n; ++d) C.F.put(o + 2 + 2 * d, iv_mul(load_tan(C, ak, ai, base, rec, d), R));
-        } break;
-        case OP_EXP:
-            for (int d = 0; d < n; ++d) C.F.put(o + 2 + 2 * d, iv_mul(V, load_tan(C, ak, ai, base, rec, d)));
-            break;
-        case OP_LOG: {
-            const iv R = iv_recip_pos(A);
-            for (int d = 0; d < n; ++d) C.F.put(o + 2 + 2 * d, iv_mul(load_tan(C, ak, ai, base, rec, d), R));
         } break;
         }
-        C.F.put(o, V);
+        C.F.to(I.y, V);
+        I = next;
     }
 }
 
-// reverse sweep of one output (reverse-mode interval AD): adjoint slots at
-// `abase` (2 units each), forward values in tape records at `tbase`, gradient
-// accumulators at `gbase`. Operand a is updated before operand b. A product
-// contribution x*y to a slot already written is accumulated with one directed
-// rounding per end (iv_fma); the first write stores the product.
-__device__ void run_reverse(const RIns* __restrict__ rins, int count, const SweepCtx& C, int abase, int tbase,
-                            int gbase) {
+// reverse sweep of one output (reverse-mode interval AD). Operand a is updated
+// before operand b. A product contribution x*y to a slot already written is
+// accumulated with one directed rounding per end (iv_fma); the first write
+// stores the product.
+__device__ __noinline__ void run_reverse(const XRIns* __restrict__ rins, int count, const SweepCtx C) {
+    const uint4* q = reinterpret_cast<const uint4*>(rins);
+    uint4 I = __ldg(q), J = __ldg(q + 1);
+    iv last = zero();   // the adjoint stored last
     for (int i = 0; i < count; ++i) {
-        const RIns R = rins[i];
-        const uint32_t op = R.w0 & 31u, wslot = R.w0 >> 16;
-        const iv W = C.F.get(abase + 2 * (int)wslot);
+        q += 2;
+        const uint4 nextI = __ldg(q), nextJ = __ldg(q + 1);
+        const uint32_t op = I.x & 31u;
+        const iv W = (I.x & kAdjLast) ? last : C.F.at(I.y);
         if (op == OP_VAR) {
-            const int g = gbase + 2 * (int)R.w1;
-            C.F.put(g, iv_add(C.F.get(g), W));
-            continue;
+            C.F.to(I.z, iv_add(C.F.at(I.z), W));
+        } else {
+            const bool a_init = (I.x >> 5) & 1u, b_init = (I.x >> 6) & 1u, a_none = (I.x >> 7) & 1u, b_none = (I.x >> 8) & 1u;
+            // contribution to operand a: W * ay (a_prod) or +-W; to operand b: bx * by or +-W
+            iv ay = W, bx = W, by = W;
+            bool prod = true;
+            switch (op) {
+            case OP_MUL:
+                if (!a_none) ay = operand(C, J.y);
+                if (!b_none) by = operand(C, J.x);
+                break;
+            case OP_DIV:
+                ay = operand(C, J.y);
+                if (!b_none) bx = iv_neg(iv_mul(W, C.F.at(J.z)));   // b gets -(W V) / B
+                break;
+            case OP_SQR:
+            case OP_SQRT: ay = iv_twice(op == OP_SQR ? operand(C, J.x) : C.F.at(J.z)); break;
+            case OP_EXP: ay = C.F.at(J.z); break;
+            case OP_LOG: ay = operand(C, J.x); break;
+            default: prod = false;
+            }
+            if (op == OP_DIV || op == OP_SQRT || op == OP_LOG) {
+                ay = op == OP_DIV || gt0(ay.lo) ? iv_recip(ay) : entire();
+                by = ay;
+            }
+            // a first contribution is fused with [0,0]: the bits of the product
+            if (!a_none) {
+                if (prod) last = iv_fma(W, ay, a_init ? zero() : C.F.at(I.z));
+                else {
+                    last = op == OP_NEG ? iv_neg(W) : W;
+                    if (!a_init) last = iv_add(C.F.at(I.z), last);
+                }
+                C.F.to(I.z, last);
+            }
+            if (!b_none) {
+                if (prod) last = iv_fma(bx, by, b_init ? zero() : C.F.at(I.w));
+                else {
+                    last = op == OP_SUB ? iv_neg(W) : W;
+                    if (!b_init) last = iv_add(C.F.at(I.w), last);
+                }
+                C.F.to(I.w, last);
+            }
         }
-        const bool a_init = (R.w0 >> 5) & 1u, b_init = (R.w0 >> 6) & 1u;
-        const bool a_none = (R.w0 >> 7) & 1u, b_none = (R.w0 >> 8) & 1u;
-        const uint32_t Ak = (R.w3 >> 16) & 3u, Bk = (R.w3 >> 18) & 3u;
-        // contribution to operand a: ax * ay (a_prod) or +-W; to operand b likewise
-        iv ax = W, ay = W, bx = W, by = W;
-        bool a_prod = true, b_prod = true, sub_b = false, sub_a = false;
-        switch (op) {
-        case OP_ADD: a_prod = b_prod = false; break;
-        case OP_SUB: a_prod = b_prod = false; sub_b = true; break;
-        case OP_NEG: a_prod = false; sub_a = true; break;
-        case OP_MUL: {
-            ay = load_val(C, Bk, R.w2 >> 16, tbase, 2);
-            by = load_val(C, Ak, R.w2 & 0xFFFFu, tbase, 2);
-        } break;
-        case OP_DIV: {
-            const iv B = load_val(C, Bk, R.w2 >> 16, tbase, 2);
-            const iv V = C.F.get(tbase + 2 * (int)(R.w3 & 0xFFFFu));
-            ay = iv_recip(B);
-            bx = iv_neg(iv_mul(W, V));            // b gets -(W V) / B
-            by = ay;
-        } break;
-        case OP_SQR: ay = iv_twice(load_val(C, Ak, R.w2 & 0xFFFFu, tbase, 2)); break;
-        case OP_SQRT: ay = iv_recip_pos(iv_twice(C.F.get(tbase + 2 * (int)(R.w3 & 0xFFFFu)))); break;
-        case OP_EXP: ay = C.F.get(tbase + 2 * (int)(R.w3 & 0xFFFFu)); break;
-        case OP_LOG: ay = iv_recip_pos(load_val(C, Ak, R.w2 & 0xFFFFu, tbase, 2)); break;
-        default: a_prod = b_prod = false; ax = bx = entire();
-        }
-        if (!a_none) {
-            const int u = abase + 2 * (int)(R.w1 & 0xFFFFu);
-            iv v;
-            if (a_prod) v = a_init ? iv_mul(ax, ay) : iv_fma(ax, ay, C.F.get(u));
-            else if (a_init) v = sub_a ? iv_neg(ax) : ax;
-            else v = sub_a ? iv_sub(C.F.get(u), ax) : iv_add(C.F.get(u), ax);
-            C.F.put(u, v);
-        }
-        if (!b_none) {
-            const int u = abase + 2 * (int)(R.w1 >> 16);
-            iv v;
-            if (b_prod) v = b_init ? iv_mul(bx, by) : iv_fma(bx, by, C.F.get(u));
-            else if (b_init) v = sub_b ? iv_neg(bx) : bx;
-            else v = sub_b ? iv_sub(C.F.get(u), bx) : iv_add(C.F.get(u), bx);
-            C.F.put(u, v);
-        }
+        I = nextI;
+        J = nextJ;
     }
 }
 
 // --------------------------------------------------------------- the kernel
 template <int MODE>
-__global__ void __launch_bounds__(512) k_bound(const KParams P) {
+__global__ void __launch_bounds__(512, 2) k_bound(const KParams P) {
     extern __shared__ double smem[];
     const ProgDesc& G = *P.prog;
     const int n = G.n, n_out = G.n_out;
     const FrameLayout L = G.L;
     SweepCtx C;
-    if (P.frame_in_smem) C.F.p = smem + threadIdx.x;
-    else C.F.p = P.gframe + (size_t)blockIdx.x * P.frame_units * blockDim.x + threadIdx.x;
-    C.F.s = blockDim.x;
+    const size_t warp = threadIdx.x >> 5;
+    if (P.frame_in_smem) C.F.p = smem + warp * P.frame_units * 32;
+    else C.F.p = P.gframe + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * P.frame_units * 32;
+    C.F.p += threadIdx.x & 31;
     C.consts = G.consts;
     C.x_base = L.x_base;
-    C.c_base = L.c_base;
 
-    tile_loop(P, [&](const Sub& s) {
+    const int groups = MODE == KM_ADJ_STORE ? P.groups : 1;
+    const int per = (int)blockDim.x / groups, first_o = MODE == KM_ADJ_STORE ? (int)threadIdx.x / per : 0;
+    tile_loop_per(P, per, [&](const Sub& s) {
         const long long g = s.g;
         const bool valid = s.valid;
         if (valid) {
@@ -245,11 +242,12 @@ __global__ void __launch_bounds__(512) k_bound(const KParams P) {
                 C.F.st(L.c_base + i, c);
             }
             // ---- Step 2a: rigorous point value f(c) of every output
-            C.point = true;
-            run_values(G.ins + G.pt_begin, G.pt_count, C, L.phase_base);
-            for (int o = 0; o < n_out; ++o)
-                C.F.put(L.fc_base + 2 * o, load_val(C, G.pt_out_kind[o], G.pt_out_ref[o], L.phase_base, 2));
-            C.point = false;
+            if (groups == 1) run_values(G.xins + G.pt_begin, G.pt_count, C);
+            for (int o = 0; o < n_out && groups == 1; ++o) {
+                const uint32_t kind = G.pt_out_kind[o], ref = G.pt_out_ref[o];
+                const double c = kind == K_VAR ? C.F.ld(L.c_base + (int)ref) : 0.0;
+                C.F.put(L.fc_base + 2 * o, kind == K_VAR ? mk(c, c) : load_val(C, kind, ref, L.phase_base, 2));
+            }
         }
         // ---- Step 2b: gradient enclosures and the Mean Value Form, output by output.
         // With the natural interval extension alone (form 1) a reduce launch needs no
@@ -259,28 +257,36 @@ __global__ void __launch_bounds__(512) k_bound(const KParams P) {
         double obj_lo = from_bits(0x7FF0000000000000LL);
         if (MODE == KM_FWD_REDUCE || MODE == KM_FWD_STORE) {
             if (valid) {
-                if (nie_only) run_values(G.ins + G.tan_begin, G.tan_count, C, L.phase_base);
-                else run_tangents(G.ins + G.tan_begin, G.tan_count, C, L.phase_base, n);
+                if (nie_only) run_values(G.xtan, G.tan_count, C);
+                else run_tangents(G.xtan, G.tan_count, C, n);
             }
         }
-        for (int o = 0; o < n_out; ++o) {
+        for (int o = first_o; o < n_out; o += groups) {
             iv F = zero(), Fc = zero();
             if (valid && nie_only) {
                 Fc = C.F.get(L.fc_base + 2 * o);
                 iv nie;
                 if (MODE == KM_FWD_REDUCE) {
-                    nie = load_val(C, G.tan_out_kind[o], G.tan_out_ref[o], L.phase_base, 2);
+                    nie = load_val(C, G.tan_out_kind[o], G.tan_out_ref[o], L.phase_base, L.tan_rec);
                 } else {
                     const AdjProgram& A = G.adj[o];
                     const int tb = L.phase_base + 2 * n + 2 * A.adj_slots;
-                    run_values(G.ins + A.fw_begin, A.fw_count, C, tb);
+                    run_values(G.xins + A.fw_begin, A.fw_count, C);
                     nie = load_val(C, A.out_kind_ref, A.out_ref, tb, 2);
                 }
                 F = final_form(1, nie, nie);
                 if (excludes_feasible(G.out_kind[o], F)) cert_infeasible = true;
                 if (o == G.obj) obj_lo = F.lo;
             } else if (valid) {
-                Fc = C.F.get(L.fc_base + 2 * o);
+                if (groups > 1) {   // f(c) of this output alone
+                    const AdjProgram& A = G.adj[o];
+                    const int tb = L.phase_base + 2 * n + 2 * A.adj_slots;
+                    run_values(G.xcone + A.fw_begin, A.fw_count, C);
+                    const double c = A.out_kind_ref == K_VAR ? C.F.ld(L.c_base + A.out_ref) : 0.0;
+                    Fc = A.out_kind_ref == K_VAR ? mk(c, c) : load_val(C, A.out_kind_ref, A.out_ref, tb, 2);
+                } else {
+                    Fc = C.F.get(L.fc_base + 2 * o);
+                }
                 iv nie;
                 int gunit, gstride;  // gradient of this output: unit of G_0 and stride (0: constant/variable)
                 if (MODE == KM_FWD_REDUCE || MODE == KM_FWD_STORE) {
@@ -292,10 +298,10 @@ __global__ void __launch_bounds__(512) k_bound(const KParams P) {
                 } else {
                     const AdjProgram& A = G.adj[o];
                     const int gb = L.phase_base, ab = gb + 2 * n, tb = ab + 2 * A.adj_slots;
-                    run_values(G.ins + A.fw_begin, A.fw_count, C, tb);
+                    run_values(G.xins + A.fw_begin, A.fw_count, C);
                     for (int i = 0; i < n; ++i) C.F.put(gb + 2 * i, zero());
                     if (A.out_wslot >= 0) C.F.put(ab + 2 * A.out_wslot, one());
-                    run_reverse(G.rins + A.rv_begin, A.rv_count, C, ab, tb, gb);
+                    run_reverse(G.xrins + A.rv_begin, A.rv_count, C);
                     nie = load_val(C, A.out_kind_ref, A.out_ref, tb, 2);
                     gunit = gb;
                     gstride = 2;
@@ -405,8 +411,7 @@ __global__ void __launch_bounds__(256) k_point_grad(const ProgDesc* __restrict__
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n_points;
          p += (long long)gridDim.x * blockDim.x) {
         Frame F;
-        F.p = gframe + (size_t)blockIdx.x * frame_units * blockDim.x + threadIdx.x;
-        F.s = blockDim.x;
+        F.p = gframe + ((size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * frame_units * 32 + (threadIdx.x & 31);
         const double* x = X + (size_t)p * n;
         for (int o = 0; o < n_out; ++o) {
             const AdjProgram& A = G.adj[o];

@@ -13,6 +13,10 @@ namespace ivb {
 struct ProgDesc {
     const Ins* ins;
     const RIns* rins;
+    const XIns* xins;
+    const XIns* xtan;
+    const XIns* xcone;
+    const XRIns* xrins;
     const double* consts;
     int32_t n, n_out, obj, has_eq;
     int32_t pt_begin, pt_count, tan_begin, tan_count;

@@ -22,6 +22,8 @@ struct ivb_problem {
     ivb::ProgDesc* d_prog = nullptr;
     ivb::Ins* d_ins = nullptr;
     ivb::RIns* d_rins = nullptr;
+    ivb::XIns* d_xins = nullptr;
+    ivb::XRIns* d_xrins = nullptr;
     double* d_consts = nullptr;
     uint8_t* d_out_kind = nullptr;
     // per-call buffers (capacity max_nodes)
