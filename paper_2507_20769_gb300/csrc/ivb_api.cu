@@ -75,31 +75,36 @@ int reduce_units(const ivb_problem* p) {
     return p->jit.state_units;
 }
 
-// Read host or device input arrays into host vectors (device arrays are
-// copied synchronously on the stream: validation needs the values).
-template <class T>
-ivb_status fetch(ivb_problem* p, const T* src, size_t count, std::vector<T>& dst, cudaStream_t s) {
-    dst.resize(count);
-    if (is_device_ptr(src)) {
-        CK(cudaMemcpyAsync(dst.data(), src, count * sizeof(T), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-    } else {
-        std::memcpy(dst.data(), src, count * sizeof(T));
-    }
-    return IVB_OK;
-}
+// staging of a call's small arrays goes through pinned memory (a pageable copy of a
+// few bytes costs some 10 us of host time each); larger calls copy directly
+constexpr size_t kPinnedMost = 1 << 20;
 
 // Validate boxes and splits, write the node queue into the pinned staging
 // buffer; returns the queue size in bytes through *bytes.
 ivb_status stage_queue(ivb_problem* p, int n_nodes, const double* boxes, const int32_t* splits, long long g_begin,
                        long long g_count, bool enclose, size_t* bytes, long long* total_out, cudaStream_t s) {
     const int n = p->n;
-    std::vector<double> B;
-    std::vector<int32_t> S;
-    ivb_status st = fetch(p, boxes, (size_t)n_nodes * n * 2, B, s);
-    if (st) return st;
-    st = fetch(p, splits, (size_t)n_nodes * n, S, s);
-    if (st) return st;
+    // host arrays are read in place; device arrays come over in two copies and one
+    // wait (validation needs the values)
+    const size_t bb = (size_t)n_nodes * n * 2 * sizeof(double), sb = (size_t)n_nodes * n * sizeof(int32_t);
+    const bool db = is_device_ptr(boxes), ds = is_device_ptr(splits);
+    std::vector<char> pageable;
+    const double* B = boxes;
+    const int32_t* S = splits;
+    if (db || ds) {
+        char* to = nullptr;
+        if (bb + sb <= kPinnedMost) {
+            const ivb_status st = ensure_pinned(p, p->h_in, bb + sb);
+            if (st) return st;
+            to = p->h_in.p;
+        } else {
+            pageable.resize(bb + sb);
+            to = pageable.data();
+        }
+        if (db) { CK(cudaMemcpyAsync(to, boxes, bb, cudaMemcpyDeviceToHost, s)); B = reinterpret_cast<double*>(to); }
+        if (ds) { CK(cudaMemcpyAsync(to + bb, splits, sb, cudaMemcpyDeviceToHost, s)); S = reinterpret_cast<int32_t*>(to + bb); }
+        CK(cudaStreamSynchronize(s));
+    }
     // the previous call's copy out of the staging buffer must have finished
     CK(cudaEventSynchronize(p->queue_free));
     char* q = p->h_queue;
@@ -115,8 +120,11 @@ ivb_status stage_queue(ivb_problem* p, int n_nodes, const double* boxes, const i
         int32_t* N = reinterpret_cast<int32_t*>(h + n);
         long long cnt = 1;
         for (int i = 0; i < n; ++i) {
-            const double a = B[((size_t)nd * n + i) * 2], b = B[((size_t)nd * n + i) * 2 + 1];
-            const int32_t k = S[(size_t)nd * n + i];
+            double ab[2];
+            int32_t k;
+            std::memcpy(ab, B + ((size_t)nd * n + i) * 2, sizeof ab);
+            std::memcpy(&k, S + (size_t)nd * n + i, sizeof k);
+            const double a = ab[0], b = ab[1];
             if (!std::isfinite(a) || !std::isfinite(b) || !(a <= b))
                 return fail(p, IVB_EINVAL, "node " + std::to_string(nd) + ": box bounds must be finite with lo <= hi");
             if (std::fabs(a) > lim || std::fabs(b) > lim)
@@ -194,8 +202,7 @@ int reduce_occupancy(ivb_problem* p, int block, int frame_smem, int tpsub = 1, b
 // enqueue: keys, counter, bound kernel, finalize (the batched graph body)
 ivb_status enqueue_bound(ivb_problem* p, int grid, int block, int tile, int frame_smem, int max_nodes, cudaStream_t s,
                          int tpsub, bool sync) {
-    CK(launch_init_keys(p->d_keys, p->d_queue, max_nodes, p->n_out, s));
-    CK(cudaMemsetAsync(p->d_counter, 0, sizeof(unsigned long long), s));
+    CK(launch_init_keys(p->d_keys, p->d_queue, max_nodes, p->n_out, p->d_counter, s));
     KParams K = make_params(p, frame_smem);
     K.tile = tile;
     CK(launch_reduce(p, K, grid, block, frame_smem, s, tpsub, sync));
@@ -207,11 +214,7 @@ ivb_status enqueue_bound(ivb_problem* p, int grid, int block, int tile, int fram
     F.obj = p->obj;
     F.filter = p->opt.filter;
     F.out_kind = p->d_out_kind;
-    F.lb = p->d_lb;
-    F.inf = p->d_inf;
-    F.ub = p->d_ub;
-    F.minlo = p->d_minlo;
-    F.maxhi = p->d_maxhi;
+    F.out_in_header = true;
     CK(launch_finalize(F, s));
     p->launches += 3;
     return IVB_OK;
@@ -399,25 +402,66 @@ ivb_status default_tuning(ivb_problem* p) {
     return IVB_OK;
 }
 
-// copy node results to the caller (device -> device or device -> host)
-ivb_status deliver(ivb_problem* p, int n_nodes, double* out_lb, uint8_t* out_inf, double* out_ub, double* out_minlo,
-                   double* out_maxhi, cudaStream_t s, bool* host_out) {
-    struct Item { void* dst; const void* src; size_t bytes; };
-    const Item items[] = {
-        {out_lb, p->d_lb, (size_t)n_nodes * sizeof(double)},
-        {out_inf, p->d_inf, (size_t)n_nodes},
-        {out_ub, p->d_ub, (size_t)n_nodes * sizeof(double)},
-        {out_minlo, p->d_minlo, (size_t)n_nodes * p->n_out * sizeof(double)},
-        {out_maxhi, p->d_maxhi, (size_t)n_nodes * p->n_out * sizeof(double)},
-    };
-    for (const Item& it : items) {
-        if (!it.dst) continue;
-        const bool dev = is_device_ptr(it.dst);
-        if (!dev) *host_out = true;
-        CK(cudaMemcpyAsync(it.dst, it.src, it.bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+// Where a call's node results go. k_finalize writes straight to device arrays of
+// this device; what the host wants is packed in d_out and comes over in one copy.
+// Anything else (another device, managed memory, an unaligned address) is copied
+// array by array.
+struct Outputs {
+    struct Item { void* user; size_t offset, bytes; bool direct, host; } it[5];
+    OutLayout L;
+    bool any_host = false;
+
+    Outputs(ivb_problem* p, int n_nodes, double* lb, uint8_t* inf, double* ub, double* minlo, double* maxhi,
+            QueueHeader* H, char* d_out)
+        : L(n_nodes, minlo || maxhi ? p->n_out : 0) {
+        const size_t n = n_nodes, hull = n * p->n_out * sizeof(double);
+        it[0] = {lb, 0, n * sizeof(double), false, false};
+        it[1] = {ub, L.ub, n * sizeof(double), false, false};
+        it[2] = {minlo, L.minlo, hull, false, false};
+        it[3] = {maxhi, L.maxhi, hull, false, false};
+        it[4] = {inf, L.inf, n, false, false};
+        void* at[5];
+        for (int k = 0; k < 5; ++k) {
+            Item& x = it[k];
+            at[k] = nullptr;
+            if (!x.user) continue;
+            cudaPointerAttributes a;
+            const bool ok = cudaPointerGetAttributes(&a, x.user) == cudaSuccess;
+            if (!ok) cudaGetLastError();
+            const bool dev = ok && (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged);
+            x.direct = dev && a.type == cudaMemoryTypeDevice && a.device == p->device &&
+                       (k == 4 || reinterpret_cast<uintptr_t>(x.user) % sizeof(double) == 0);
+            x.host = !dev;
+            any_host |= x.host;
+            at[k] = x.direct ? x.user : d_out + x.offset;
+        }
+        H->lb = static_cast<double*>(at[0]);
+        H->ub = static_cast<double*>(at[1]);
+        H->minlo = static_cast<double*>(at[2]);
+        H->maxhi = static_cast<double*>(at[3]);
+        H->inf = static_cast<uint8_t*>(at[4]);
     }
-    return IVB_OK;
-}
+
+    // after the kernels are enqueued: copies, and the wait that host arrays need
+    ivb_status deliver(ivb_problem* p, const char* d_out, cudaStream_t s) const {
+        const bool packed = any_host && L.bytes <= kPinnedMost;
+        if (packed) {
+            const ivb_status st = ensure_pinned(p, p->h_out, L.bytes);
+            if (st) return st;
+            CK(cudaMemcpyAsync(p->h_out.p, d_out, L.bytes, cudaMemcpyDeviceToHost, s));
+        }
+        for (const Item& x : it) {
+            if (!x.user || x.direct || (x.host && packed)) continue;
+            CK(cudaMemcpyAsync(x.user, d_out + x.offset, x.bytes, x.host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, s));
+        }
+        if (!any_host) return IVB_OK;
+        CK(cudaStreamSynchronize(s));
+        if (packed)
+            for (const Item& x : it)
+                if (x.user && x.host) std::memcpy(x.user, p->h_out.p + x.offset, x.bytes);
+        return IVB_OK;
+    }
+};
 
 }  // namespace
 
@@ -638,11 +682,7 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     CKC(cudaEventRecord(p->queue_free, 0));
     CKC(cudaMalloc(&p->d_keys, (size_t)p->max_nodes * (2 * p->n_out + 2) * sizeof(unsigned long long)));
     CKC(cudaMalloc(&p->d_counter, sizeof(unsigned long long)));
-    CKC(cudaMalloc(&p->d_lb, (size_t)p->max_nodes * sizeof(double)));
-    CKC(cudaMalloc(&p->d_ub, (size_t)p->max_nodes * sizeof(double)));
-    CKC(cudaMalloc(&p->d_inf, (size_t)p->max_nodes));
-    CKC(cudaMalloc(&p->d_minlo, (size_t)p->max_nodes * p->n_out * sizeof(double)));
-    CKC(cudaMalloc(&p->d_maxhi, (size_t)p->max_nodes * p->n_out * sizeof(double)));
+    CKC(cudaMalloc(&p->d_out, OutLayout(p->max_nodes, p->n_out).bytes));
     CKC(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
     if (o.specialize) {
         const int64_t* cnt = o.grad_mode == IVB_GRAD_ADJOINT ? p->P.cnt_adj : p->P.cnt_fwd;
@@ -673,29 +713,40 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     return IVB_OK;
 }
 
+ivb_status ensure_pinned(ivb_problem* p, ivb_problem::Pinned& P, size_t bytes) {
+    if (bytes <= P.bytes) return IVB_OK;
+    if (P.p) cudaFreeHost(P.p);
+    P.p = nullptr;
+    P.bytes = 0;
+    const size_t want = std::max<size_t>(2 * bytes, 4096);
+    CK(cudaMallocHost(&P.p, want));
+    P.bytes = want;
+    return IVB_OK;
+}
+
 namespace {
 ivb_status bound_nodes_impl(ivb_problem* p, int32_t n_nodes, const double* boxes, const int32_t* splits_per_dim,
                             double* out_lb, uint8_t* out_infeasible, double* out_ub, double* out_minlo,
-                            double* out_maxhi, cudaStream_t s, bool wait_host);
+                            double* out_maxhi, char* packed, cudaStream_t s);
 }  // namespace
 
 extern "C" ivb_status ivb_bound_nodes_ex(ivb_problem* p, int32_t n_nodes, const double* boxes,
                                          const int32_t* splits_per_dim, double* out_lb, uint8_t* out_infeasible,
                                          double* out_ub, double* out_minlo, double* out_maxhi, void* cuda_stream) {
     return bound_nodes_impl(p, n_nodes, boxes, splits_per_dim, out_lb, out_infeasible, out_ub, out_minlo, out_maxhi,
-                            (cudaStream_t)cuda_stream, true);
+                            nullptr, (cudaStream_t)cuda_stream);
 }
 
 ivb_status bound_nodes_enqueue(ivb_problem* p, int32_t n_nodes, const double* boxes, const int32_t* splits,
-                               double* out_lb, uint8_t* out_inf, double* out_ub, double* out_minlo,
-                               double* out_maxhi, cudaStream_t s) {
-    return bound_nodes_impl(p, n_nodes, boxes, splits, out_lb, out_inf, out_ub, out_minlo, out_maxhi, s, false);
+                               char* packed, cudaStream_t s) {
+    return bound_nodes_impl(p, n_nodes, boxes, splits, nullptr, nullptr, nullptr, nullptr, nullptr, packed, s);
 }
 
 namespace {
+// packed: results of the nodes go there in one copy, without a wait (bound_nodes_enqueue)
 ivb_status bound_nodes_impl(ivb_problem* p, int32_t n_nodes, const double* boxes, const int32_t* splits_per_dim,
                             double* out_lb, uint8_t* out_infeasible, double* out_ub, double* out_minlo,
-                            double* out_maxhi, cudaStream_t s, bool wait_host) {
+                            double* out_maxhi, char* packed, cudaStream_t s) {
     if (!p) return fail(nullptr, IVB_EINVAL, "problem handle is NULL");
     p->err.clear();
     if (n_nodes == 0) return IVB_OK;   // empty batch: nothing to bound
@@ -706,7 +757,14 @@ ivb_status bound_nodes_impl(ivb_problem* p, int32_t n_nodes, const double* boxes
     long long total = 0;
     ivb_status st = stage_queue(p, n_nodes, boxes, splits_per_dim, 0, 0, false, &qbytes, &total, s);
     if (st) return st;
-    bool host_out = false;
+    QueueHeader* H = reinterpret_cast<QueueHeader*>(p->h_queue);
+    const Outputs out(p, n_nodes, out_lb, out_infeasible, out_ub, out_minlo, out_maxhi, H, p->d_out);
+    if (packed) {
+        const OutLayout L(n_nodes, 0);
+        H->lb = reinterpret_cast<double*>(p->d_out);
+        H->ub = reinterpret_cast<double*>(p->d_out + L.ub);
+        H->inf = reinterpret_cast<uint8_t*>(p->d_out + L.inf);
+    }
 
     if (!p->opt.batched) {
         // plain path: one node per launch, node queue of one record each
@@ -730,16 +788,18 @@ ivb_status bound_nodes_impl(ivb_problem* p, int32_t n_nodes, const double* boxes
             const int grid = (int)std::min<long long>(tiles, (long long)p->sm_count * p->bps);
             if (reduce_units(p) > 0) st = ensure_frame(p, grid, p->block, reduce_units(p));
             if (st) return st;
-            CK(launch_init_keys(p->d_keys, p->d_queue, 1, p->n_out, s));
-            CK(cudaMemsetAsync(p->d_counter, 0, sizeof(unsigned long long), s));
+            CK(launch_init_keys(p->d_keys, p->d_queue, 1, p->n_out, p->d_counter, s));
             KParams K = make_params(p, p->frame_smem);
             K.tile = pass_size(p, p->block, p->tpsub);
             CK(launch_reduce(p, K, grid, p->block, p->frame_smem, s, p->tpsub, p->chunk_sync));
             FinalizeParams F{};
             F.keys = p->d_keys; F.queue = p->d_queue; F.max_nodes = 1; F.n_out = p->n_out; F.obj = p->obj;
             F.filter = p->opt.filter; F.out_kind = p->d_out_kind;
-            F.lb = p->d_lb + nd; F.inf = p->d_inf + nd; F.ub = p->d_ub + nd;
-            F.minlo = p->d_minlo + (size_t)nd * p->n_out; F.maxhi = p->d_maxhi + (size_t)nd * p->n_out;
+            if (H->lb) F.lb = H->lb + nd;
+            if (H->inf) F.inf = H->inf + nd;
+            if (H->ub) F.ub = H->ub + nd;
+            if (H->minlo) F.minlo = H->minlo + (size_t)nd * p->n_out;
+            if (H->maxhi) F.maxhi = H->maxhi + (size_t)nd * p->n_out;
             CK(launch_finalize(F, s));
             p->launches += 3;
             // the host buffer `one` is reused: wait for this node's copy
@@ -782,10 +842,11 @@ ivb_status bound_nodes_impl(ivb_problem* p, int32_t n_nodes, const double* boxes
             if (st) return st;
         }
     }
-    st = deliver(p, n_nodes, out_lb, out_infeasible, out_ub, out_minlo, out_maxhi, s, &host_out);
-    if (st) return st;
-    if (host_out && wait_host) CK(cudaStreamSynchronize(s));
-    return IVB_OK;
+    if (packed) {
+        CK(cudaMemcpyAsync(packed, p->d_out, OutLayout(n_nodes, 0).bytes, cudaMemcpyDeviceToHost, s));
+        return IVB_OK;
+    }
+    return out.deliver(p, p->d_out, s);
 }
 }  // namespace
 
@@ -1082,11 +1143,9 @@ extern "C" void ivb_destroy(ivb_problem* p) {
     if (p->h_queue) cudaFreeHost(p->h_queue);
     cudaFree(p->d_keys);
     cudaFree(p->d_counter);
-    cudaFree(p->d_lb);
-    cudaFree(p->d_ub);
-    cudaFree(p->d_inf);
-    cudaFree(p->d_minlo);
-    cudaFree(p->d_maxhi);
+    cudaFree(p->d_out);
+    for (ivb_problem::Pinned* P : {&p->h_in, &p->h_out, &p->h_bnb[0], &p->h_bnb[1]})
+        if (P->p) cudaFreeHost(P->p);
     cudaFree(p->d_frame);
     cudaFree(p->d_pframe);
     jit_unload(p->jit);

@@ -46,9 +46,10 @@ struct Batch {
     std::vector<Node*> kids;
     std::vector<double> boxes;
     std::vector<int32_t> splits;
-    double* lb = nullptr;
-    double* ub = nullptr;
-    uint8_t* inf = nullptr;
+    char* packed = nullptr;        // OutLayout of the batch's nodes
+    const double* lb = nullptr;
+    const double* ub = nullptr;
+    const uint8_t* inf = nullptr;
     cudaEvent_t done = nullptr;
     double parent_lb = INFINITY;   // smallest lower bound of the parents (open while in flight)
     bool in_flight = false;
@@ -138,20 +139,19 @@ extern "C" ivb_status ivb_bnb_solve(ivb_problem* p, int32_t n, const double* roo
     for (Batch& b : bat) {
         b.boxes.resize((size_t)cap * n * 2);
         b.splits.resize((size_t)cap * n);
-        if (cudaMallocHost(&b.lb, cap * sizeof(double)) != cudaSuccess ||
-            cudaMallocHost(&b.ub, cap * sizeof(double)) != cudaSuccess ||
-            cudaMallocHost(&b.inf, cap) != cudaSuccess ||
+        const int k = (int)(&b - bat);
+        if (st || (o->overlap == 0 && k > 0)) continue;
+        // pinned results, kept by the problem for its next search
+        if (ensure_pinned(p, p->h_bnb[k], OutLayout(cap, 0).bytes) != IVB_OK ||
             cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming) != cudaSuccess)
             st = IVB_ENOMEM;
+        b.packed = p->h_bnb[k].p;
     }
     auto release = [&]() {
         for (Batch& b : bat) {
             if (b.in_flight && b.done) cudaEventSynchronize(b.done);
             for (Node* k : b.kids) delete k;
             b.kids.clear();
-            if (b.lb) cudaFreeHost(b.lb);
-            if (b.ub) cudaFreeHost(b.ub);
-            if (b.inf) cudaFreeHost(b.inf);
             if (b.done) cudaEventDestroy(b.done);
         }
         while (!heap.empty()) { delete heap.top(); heap.pop(); }
@@ -192,8 +192,11 @@ extern "C" ivb_status ivb_bnb_solve(ivb_problem* p, int32_t n, const double* roo
             subs += s;
         }
         bounded += cnt;
-        ivb_status e = bound_nodes_enqueue(p, cnt, b.boxes.data(), b.splits.data(), b.lb, b.inf, b.ub, nullptr,
-                                           nullptr, stream);
+        const OutLayout L(cnt, 0);
+        b.lb = reinterpret_cast<const double*>(b.packed);
+        b.ub = reinterpret_cast<const double*>(b.packed + L.ub);
+        b.inf = reinterpret_cast<const uint8_t*>(b.packed + L.inf);
+        ivb_status e = bound_nodes_enqueue(p, cnt, b.boxes.data(), b.splits.data(), b.packed, stream);
         if (e) return e;
         if (cudaEventRecord(b.done, stream) != cudaSuccess) return IVB_ECUDA;
         b.in_flight = true;

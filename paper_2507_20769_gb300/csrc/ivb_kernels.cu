@@ -355,7 +355,8 @@ __global__ void __launch_bounds__(512, 2) k_bound(const KParams P) {
 namespace ivb {
 
 // ------------------------------------------------------------ node results
-__global__ void k_init_keys(unsigned long long* keys, const char* queue, int n_out) {
+__global__ void k_init_keys(unsigned long long* keys, const char* queue, int n_out, unsigned long long* counter) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0ULL;
     const int n_nodes = (int)reinterpret_cast<const long long*>(queue)[0];
     const int K = 2 * n_out + 2;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes * K; i += gridDim.x * blockDim.x) {
@@ -368,7 +369,11 @@ __global__ void k_init_keys(unsigned long long* keys, const char* queue, int n_o
 // Section 3.1 Step 3 and pruning: lb = lower end of the objective's
 // refinement (or the filtered minimum), infeasible when an inequality's lower
 // end is > 0 or an equality's refinement excludes 0.
-__global__ void k_finalize(const FinalizeParams F) {
+__global__ void k_finalize(FinalizeParams F) {
+    if (F.out_in_header) {
+        const QueueHeader& H = *reinterpret_cast<const QueueHeader*>(F.queue);
+        F.lb = H.lb; F.inf = H.inf; F.ub = H.ub; F.minlo = H.minlo; F.maxhi = H.maxhi;
+    }
     const int nd = blockIdx.x * blockDim.x + threadIdx.x;
     const int n_nodes = (int)reinterpret_cast<const long long*>(F.queue)[0];
     if (nd >= n_nodes) return;
@@ -655,10 +660,11 @@ cudaError_t launch_bound(int mode, const KParams& P, int grid, int block, size_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_init_keys(unsigned long long* keys, const char* queue, int max_nodes, int n_out, cudaStream_t s) {
+cudaError_t launch_init_keys(unsigned long long* keys, const char* queue, int max_nodes, int n_out,
+                             unsigned long long* counter, cudaStream_t s) {
     const int total = max_nodes * (2 * n_out + 2);
     const int block = 256, grid = (total + block - 1) / block < 1024 ? (total + block - 1) / block : 1024;
-    k_init_keys<<<grid, block, 0, s>>>(keys, queue, n_out);
+    k_init_keys<<<grid, block, 0, s>>>(keys, queue, n_out, counter);
     return cudaGetLastError();
 }
 

@@ -38,6 +38,7 @@ struct FinalizeParams {
     const unsigned long long* keys;
     const char* queue;     // n_nodes is read from the queue header
     int32_t max_nodes, n_out, obj, filter;
+    bool out_in_header;    // the result arrays below are named in the queue header instead
     const uint8_t* out_kind;
     double* lb;
     uint8_t* inf;
@@ -48,7 +49,9 @@ struct FinalizeParams {
 
 cudaError_t launch_bound(int mode, const KParams& P, int grid, int block, size_t smem, cudaStream_t s);
 cudaError_t set_bound_smem_limit(int mode, int bytes);
-cudaError_t launch_init_keys(unsigned long long* keys, const char* queue, int max_nodes, int n_out, cudaStream_t s);
+// neutral keys for the queue's nodes, and the work counter to 0
+cudaError_t launch_init_keys(unsigned long long* keys, const char* queue, int max_nodes, int n_out,
+                             unsigned long long* counter, cudaStream_t s);
 cudaError_t launch_finalize(const FinalizeParams& F, cudaStream_t s);
 cudaError_t launch_point_grad(const ProgDesc* prog, int n, int n_out, int frame_units, long long n_points,
                               const double* x, double* f, double* grad, double* gframe, int grid, int block,

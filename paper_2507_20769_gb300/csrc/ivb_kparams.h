@@ -13,12 +13,23 @@ enum KernelMode { KM_FWD_REDUCE = 0, KM_ADJ_REDUCE = 1, KM_FWD_STORE = 2, KM_ADJ
 
 // Device node queue, one contiguous buffer written by a single host->device
 // copy per call:
-//   header   : int64 n_nodes, int64 g_end (end of the global index range)
-//              padded to 64 bytes
+//   header   : QueueHeader, 64 bytes: node count, end of the global index
+//              range, and where k_finalize writes the node results (they
+//              travel with the queue, so a replayed graph needs no new
+//              parameters)
 //   off      : int64 [n_nodes + 1], exclusive prefix sums of subdomain counts
 //   records  : n_nodes records of rec_bytes: double lo[n], hi[n], h[n] with
 //              h = RN(RN(hi - lo) / N), then int32 N[n]
 constexpr int kQueueHeader = 64;
+struct QueueHeader {
+    long long n_nodes, g_end;
+    double* lb;
+    uint8_t* inf;
+    double* ub;
+    double* minlo;
+    double* maxhi;
+    long long pad;
+};
 
 struct ProgDesc;
 

@@ -34,8 +34,10 @@ struct ivb_problem {
     cudaEvent_t queue_free = nullptr;   // the last copy out of h_queue has completed
     unsigned long long* d_keys = nullptr;
     unsigned long long* d_counter = nullptr;
-    double *d_lb = nullptr, *d_ub = nullptr, *d_minlo = nullptr, *d_maxhi = nullptr;
-    uint8_t* d_inf = nullptr;
+    char* d_out = nullptr;              // node results of a call, packed (OutLayout), max_nodes capacity
+    // pinned staging, kept while small: device inputs on their way to the queue,
+    // packed node results on their way to host arrays, B&B batches
+    struct Pinned { char* p = nullptr; size_t bytes = 0; } h_in, h_out, h_bnb[2];
     // frames
     double* d_frame = nullptr;
     size_t frame_bytes = 0;
@@ -61,8 +63,16 @@ struct ivb_problem {
     std::string err;
 };
 
-// ivb_bound_nodes_ex without the final wait: results reach host buffers
-// asynchronously (pinned buffers for true overlap); the caller orders on `s`
+// node results of n nodes packed in one buffer: lb, ub, minlo, maxhi, infeasible
+struct OutLayout {
+    size_t ub, minlo, maxhi, inf, bytes;   // byte offsets (lb at 0)
+    OutLayout(size_t n, size_t n_out)
+        : ub(8 * n), minlo(16 * n), maxhi(16 * n + 8 * n * n_out), inf(16 * n + 16 * n * n_out), bytes(inf + n) {}
+};
+// ivb_bound_nodes_ex on host arrays without the final wait: lb, ub and flags of
+// the nodes reach the pinned buffer `packed` (OutLayout(n_nodes, 0)) in one
+// copy; the caller orders on `s`
 ivb_status bound_nodes_enqueue(ivb_problem* p, int32_t n_nodes, const double* boxes, const int32_t* splits,
-                               double* out_lb, uint8_t* out_inf, double* out_ub, double* out_minlo,
-                               double* out_maxhi, cudaStream_t s);
+                               char* packed, cudaStream_t s);
+// at least `bytes` of pinned memory in P (grown, not shrunk); freed with the problem
+ivb_status ensure_pinned(ivb_problem* p, ivb_problem::Pinned& P, size_t bytes);

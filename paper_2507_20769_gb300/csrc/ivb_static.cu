@@ -162,13 +162,12 @@ extern "C" ivb_status ivb_bound_nodes_noalloc(ivb_problem* p, int32_t n_nodes, c
     unsigned long long* errw = reinterpret_cast<unsigned long long*>(base + kErrorOff);
     cudaStream_t s = (cudaStream_t)cuda_stream;
 
-    // what must start at a fixed value: work counter 0, error word "no error"
-    CKN(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s));
+    // what must start at a fixed value: error word "no error" (the keys and the work counter: k_init_keys)
     CKN(cudaMemsetAsync(errw, 0xFF, sizeof(unsigned long long), s));
     const int rec = queue_rec_bytes(p->n);
     k_prepare_queue<<<1, 256, 0, s>>>(boxes, splits_per_dim, n_nodes, p->n, rec, queue, errw);
     CKN(cudaGetLastError());
-    CKN(launch_init_keys(keys, queue, n_nodes, p->n_out, s));
+    CKN(launch_init_keys(keys, queue, n_nodes, p->n_out, counter, s));
     KParams K{};
     K.prog = p->d_prog;
     K.queue = queue;
