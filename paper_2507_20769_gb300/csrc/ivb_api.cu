@@ -631,25 +631,27 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     for (int m = 0; m < 4; ++m) CKC(set_bound_smem_limit(m, p->smem_optin - 1024));
     CKC(init_math_tables());
 
-    CKC(cudaMalloc(&p->d_ins, std::max<size_t>(1, ins.size()) * sizeof(Ins)));
-    CKC(cudaMalloc(&p->d_rins, std::max<size_t>(1, rins.size()) * sizeof(RIns)));
     CKC(cudaMalloc(&p->d_consts, std::max<size_t>(1, consts.size()) * sizeof(double)));
-    if (!ins.empty()) CKC(cudaMemcpy(p->d_ins, ins.data(), ins.size() * sizeof(Ins), cudaMemcpyHostToDevice));
-    if (!rins.empty()) CKC(cudaMemcpy(p->d_rins, rins.data(), rins.size() * sizeof(RIns), cudaMemcpyHostToDevice));
     if (!consts.empty())
         CKC(cudaMemcpy(p->d_consts, consts.data(), consts.size() * sizeof(double), cudaMemcpyHostToDevice));
-    std::vector<XIns> xins;
-    std::vector<XRIns> xrins;
+    std::vector<XIns> xins, pins;
+    std::vector<XRIns> xrins, prins;
     interpreter_programs(p->P, ins, rins, xins, xrins);
     CKC(cudaMalloc(&p->d_xins, xins.size() * sizeof(XIns)));
     CKC(cudaMalloc(&p->d_xrins, xrins.size() * sizeof(XRIns)));
     CKC(cudaMemcpy(p->d_xins, xins.data(), xins.size() * sizeof(XIns), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(p->d_xrins, xrins.data(), xrins.size() * sizeof(XRIns), cudaMemcpyHostToDevice));
+    const size_t xtan = ins.size();
+    p->point_units = point_programs(p->P, ins, rins, pins, prins);
+    CKC(cudaMalloc(&p->d_pins, pins.size() * sizeof(XIns)));
+    CKC(cudaMalloc(&p->d_prins, prins.size() * sizeof(XRIns)));
+    CKC(cudaMemcpy(p->d_pins, pins.data(), pins.size() * sizeof(XIns), cudaMemcpyHostToDevice));
+    CKC(cudaMemcpy(p->d_prins, prins.data(), prins.size() * sizeof(XRIns), cudaMemcpyHostToDevice));
     ProgDesc D{};
-    D.ins = p->d_ins;
-    D.rins = p->d_rins;
+    D.pins = p->d_pins;
+    D.prins = p->d_prins;
     D.xins = p->d_xins;
-    D.xtan = p->d_xins + ins.size();
+    D.xtan = p->d_xins + xtan;
     D.xcone = D.xtan + p->P.tan_count;
     D.xrins = p->d_xrins;
     D.consts = p->d_consts;
@@ -929,12 +931,9 @@ extern "C" ivb_status ivb_point_grad(ivb_problem* p, int64_t n_points, const dou
     if (!dx) { CK(cudaMallocAsync(&tx, xb, s)); CK(cudaMemcpyAsync(tx, x, xb, cudaMemcpyHostToDevice, s)); }
     if (!df) CK(cudaMallocAsync(&tf, fb, s));
     if (out_grad && !dg) CK(cudaMallocAsync(&tg, gb, s));
-    int units = 0;
-    for (int o = 0; o < n_out; ++o)
-        units = std::max(units, n + p->P.adj[o].adj_slots + p->P.adj[o].tape_records);
-    const int block = 128;
-    const int grid = (int)std::min<long long>((n_points + block - 1) / block, (long long)p->sm_count * 8);
-    const size_t need = (size_t)grid * block * std::max(units, 1) * sizeof(double);
+    const int units = p->point_units, block = 64;   // small blocks spread few points evenly
+    const int grid = (int)std::min<long long>((n_points + block - 1) / block, (long long)p->sm_count * 16);
+    const size_t need = (size_t)grid * block * units * sizeof(double);
     if (need > p->pframe_bytes) {
         if (p->d_pframe) CK(cudaFree(p->d_pframe));
         p->d_pframe = nullptr;
@@ -942,7 +941,7 @@ extern "C" ivb_status ivb_point_grad(ivb_problem* p, int64_t n_points, const dou
         CK(cudaMalloc(&p->d_pframe, need));
         p->pframe_bytes = need;
     }
-    CK(launch_point_grad(p->d_prog, n, n_out, std::max(units, 1), n_points, dx ? x : tx, df ? out_f : tf,
+    CK(launch_point_grad(p->d_prog, n, n_out, units, n_points, dx ? x : tx, df ? out_f : tf,
                          out_grad ? (dg ? out_grad : tg) : nullptr, p->d_pframe, grid, block, s));
     p->launches += 1;
     if (!df) CK(cudaMemcpyAsync(out_f, tf, fb, cudaMemcpyDeviceToHost, s));
@@ -1133,10 +1132,10 @@ extern "C" void ivb_destroy(ivb_problem* p) {
     if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
     if (p->queue_free) { cudaEventSynchronize(p->queue_free); cudaEventDestroy(p->queue_free); }
     cudaFree(p->d_prog);
-    cudaFree(p->d_ins);
-    cudaFree(p->d_rins);
     cudaFree(p->d_xins);
     cudaFree(p->d_xrins);
+    cudaFree(p->d_pins);
+    cudaFree(p->d_prins);
     cudaFree(p->d_consts);
     cudaFree(p->d_out_kind);
     cudaFree(p->d_queue);

@@ -401,4 +401,52 @@ void interpreter_programs(const HostProgram& P, const std::vector<Ins>& ins, con
     }
 }
 
+int point_programs(const HostProgram& P, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
+                   std::vector<XIns>& xins, std::vector<XRIns>& xrins) {
+    const int n = P.n_vars;
+    int units = 2 * n + 1;
+    xins.assign(ins.size() + 1, XIns{});
+    xrins.assign(rins.size() + 1, XRIns{});
+    for (int o = 0; o < P.n_out; ++o) {
+        const AdjProgram& A = P.adj[o];
+        const int gb = n, ab = 2 * n, tb = ab + A.adj_slots;
+        units = std::max(units, tb + A.tape_records);
+        auto word = [&](uint32_t kind, uint32_t idx) -> uint32_t {
+            if (kind == K_CONST) return idx | kOpConst;
+            return (uint32_t)(kind == K_VAR ? (int)idx : tb + (int)idx) * 32u;
+        };
+        uint32_t last = ~0u;
+        for (int i = A.fw_begin; i < A.fw_begin + A.fw_count; ++i) {
+            const Ins& I = ins[i];
+            const uint32_t ak = (I.w0 >> 5) & 3u, bk = (I.w0 >> 7) & 3u;
+            XIns& X = xins[i];
+            X.w = I.w0 & 31u;
+            X.dst = word(K_SLOT, I.w0 >> 16);
+            X.a = word(ak, I.w1 & 0xFFFFu);
+            X.b = bk == K_NONE ? X.a : word(bk, I.w1 >> 16);
+            if (X.a == last) X.a |= kOpLast;
+            if (X.b == last) X.b |= kOpLast;
+            last = X.dst;
+        }
+        last = ~0u;
+        for (int i = A.rv_begin; i < A.rv_begin + A.rv_count; ++i) {
+            const RIns& R = rins[i];
+            XRIns& X = xrins[i];
+            auto slot = [&](uint32_t k) { return (uint32_t)(ab + (int)k) * 32u; };
+            X.w = R.w0 & 0x1FFu;
+            X.slot = slot(R.w0 >> 16);
+            if (X.slot == last) X.w |= kAdjLast;
+            if ((R.w0 & 31u) == OP_VAR) { X.a_adj = (uint32_t)(gb + (int)R.w1) * 32u; continue; }
+            X.a_adj = slot(R.w1 & 0xFFFFu);
+            X.b_adj = slot(R.w1 >> 16);
+            if (!((R.w0 >> 8) & 1u)) last = X.b_adj;
+            else if (!((R.w0 >> 7) & 1u)) last = X.a_adj;
+            X.A = word((R.w3 >> 16) & 3u, R.w2 & 0xFFFFu);
+            X.B = word((R.w3 >> 18) & 3u, R.w2 >> 16);
+            X.V = word(K_SLOT, R.w3 & 0xFFFFu);
+        }
+    }
+    return units;
+}
+
 }  // namespace ivb

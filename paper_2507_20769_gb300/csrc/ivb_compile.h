@@ -24,4 +24,10 @@ std::string compile_tape(const ivb_tape* t, HostProgram& P, std::vector<Ins>& in
 void interpreter_programs(const HostProgram& P, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
                           std::vector<XIns>& xins, std::vector<XRIns>& xrins);
 
+// the point gradients' form of the outputs' programs, entry by entry beside `ins`
+// and `rins`: one frame unit per value, x_i at unit i, then G_i, the adjoints and
+// the tape of the output; returns the frame units
+int point_programs(const HostProgram& P, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
+                   std::vector<XIns>& xins, std::vector<XRIns>& xrins);
+
 }  // namespace ivb

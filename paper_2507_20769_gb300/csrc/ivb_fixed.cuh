@@ -72,16 +72,30 @@ __device__ __forceinline__ fx64 rcp62(fx64 Y) {
 __device__ __forceinline__ fx64 settle(fx64 q, long long rem, bool away) {
     return away ? q + (rem > 0 ? 1 : 0) : q - (rem < 0 ? 1 : 0);
 }
+// the nearest significand instead; one unit of q changes the remainder by d
+// (neither quotients nor roots of 53-bit significands are halfway between two)
+__device__ __forceinline__ fx64 settle_near(fx64 q, long long rem, long long d) {
+    return q + (2 * rem > d ? 1 : 0) - (-2 * rem > d ? 1 : 0);
+}
 
 __device__ __forceinline__ int bexp(double x) { return (int)((bits(x) >> 52) & 0x7FF); }
 
 // 1 / |y| for y normal with a normal reciprocal; away: toward +inf
 __device__ __forceinline__ bool rcp_fits(double y) { return (fx32)(bexp(y) - 1) < 2044u; }
-__device__ __forceinline__ fx64 rcp_mag(double y, bool away) {
-    const fx64 Y = sig53(y);
+__device__ __forceinline__ fx64 rcp_sig(fx64 Y, long long* rem) {
     const fx64 q = rcp62(Y) >> 9;                          // units of 2^-53
-    const long long rem = -(long long)(Y * q);             // 2^105 - Y q
+    *rem = -(long long)(Y * q);                            // 2^105 - Y q
+    return q;
+}
+__device__ __forceinline__ fx64 rcp_mag(double y, bool away) {
+    long long rem;
+    const fx64 q = rcp_sig(sig53(y), &rem);
     return settle(q, rem, away) + ((fx64)(fx32)(2044 - bexp(y)) << 52);
+}
+__device__ __forceinline__ fx64 rcp_near(double y) {
+    long long rem;
+    const fx64 Y = sig53(y), q = rcp_sig(Y, &rem);
+    return settle_near(q, rem, (long long)Y) + ((fx64)(fx32)(2044 - bexp(y)) << 52);
 }
 
 // |x| / |y| for normal x and y with |Ex - Ey| <= 1000; r62 = rcp62(sig53(y))
@@ -94,21 +108,31 @@ __device__ __forceinline__ fx64 mulhi64_near(fx64 a, fx64 b) {
     const fx64 m = wide(hi32(a), lo32(b)), n = wide(lo32(a), hi32(b));
     return wide(hi32(a), hi32(b)) + hi32(m) + hi32(n);
 }
-__device__ __forceinline__ fx64 div_mag(double x, double y, fx64 r62, bool away) {
-    const fx64 X = sig53(x), Y = sig53(y);
+__device__ __forceinline__ fx64 div_sig(fx64 X, fx64 Y, fx64 r62, int* big, long long* rem) {
     const fx64 h = mulhi64_near(X << 11, r62 + 4);         // x / y in units of 2^-61, too large by 1 to 14
-    const int big = (int)(h >> 61);                        // quotient >= 1
-    const fx64 q = h >> (8 + big);
-    const long long rem = (long long)((X << (53 - big)) - Y * q);
+    *big = (int)(h >> 61);                                 // quotient >= 1
+    const fx64 q = h >> (8 + *big);
+    *rem = (long long)((X << (53 - *big)) - Y * q);
+    return q;
+}
+__device__ __forceinline__ fx64 div_mag(double x, double y, fx64 r62, bool away) {
+    int big;
+    long long rem;
+    const fx64 q = div_sig(sig53(x), sig53(y), r62, &big, &rem);
     return settle(q, rem, away) + ((fx64)(fx32)(bexp(x) - bexp(y) + 1021 + big) << 52);
+}
+__device__ __forceinline__ fx64 div_near(double x, double y) {
+    int big;
+    long long rem;
+    const fx64 Y = sig53(y), q = div_sig(sig53(x), Y, rcp62(Y), &big, &rem);
+    return settle_near(q, rem, (long long)Y) + ((fx64)(fx32)(bexp(x) - bexp(y) + 1021 + big) << 52);
 }
 
 // sqrt of a normal x > 0. g0 = a r0 (32 bits, r0 the seed cut below
 // 1/sqrt(a)), d = a - g0^2 exactly, then c = d r0 / 2 and the second order
 // c (eta - c r0 / 2) with eta = 1 - g0 r0; the third is below 2^-56.
 __device__ __forceinline__ bool sqrt_fits(double x) { return (fx32)((bits(x) >> 52) - 1) < 2046u; }
-__device__ __forceinline__ fx64 sqrt_mag(double x, bool up) {
-    const int E = bexp(x), odd = (E + 1) & 1;
+__device__ __forceinline__ fx64 sqrt_sig(double x, int odd, long long* rem) {
     const fx64 Y = sig53(x), A = Y << odd;                 // a in [1, 4) in units of 2^-52
     const fx32 R0 = unit24(rsqrt_approx_f(__int_as_float(((127 + odd) << 23) | top23(Y)))) - 4;
     const fx64 ar = wide(hi32(A), R0) + __umulhi(lo32(A), R0);   // a r0, 2^-44
@@ -120,8 +144,21 @@ __device__ __forceinline__ fx64 sqrt_mag(double x, bool up) {
     const fx32 w = eta - (__umulhi(cq, R0 << 7) >> 1);     // eta - c r0 / 2, 2^-47
     const fx64 s = ((fx64)G << 31) + c + (__umulhi(cq, w) >> 1) + 512;   // 2^-62
     const fx64 q = s >> 10;
-    const long long rem = (long long)((A << 52) - q * q);
-    return settle(q, rem, up) + ((fx64)(fx32)((E - 1023 - odd) / 2 + 1022) << 52);
+    *rem = (long long)((A << 52) - q * q);
+    return q;
+}
+__device__ __forceinline__ fx64 sqrt_exponent(int E, int odd) { return (fx64)(fx32)((E - 1023 - odd) / 2 + 1022) << 52; }
+__device__ __forceinline__ fx64 sqrt_mag(double x, bool up) {
+    const int E = bexp(x), odd = (E + 1) & 1;
+    long long rem;
+    const fx64 q = sqrt_sig(x, odd, &rem);
+    return settle(q, rem, up) + sqrt_exponent(E, odd);
+}
+__device__ __forceinline__ fx64 sqrt_near(double x) {   // (q + 1/2)^2 - q^2 = q + 1/4
+    const int E = bexp(x), odd = (E + 1) & 1;
+    long long rem;
+    const fx64 q = sqrt_sig(x, odd, &rem);
+    return q + (rem > (long long)q ? 1 : 0) - (-rem >= (long long)q ? 1 : 0) + sqrt_exponent(E, odd);
 }
 
 // exp(x) rounded outward, |x| <= 700. With L = ln2 / 512 and k = floor(x / L)
@@ -131,7 +168,7 @@ __device__ __forceinline__ fx64 sqrt_mag(double x, bool up) {
 __device__ __forceinline__ bool exp_fits(double x) {
     return (fx32)hi32((fx64)bits(x) & 0x7FFFFFFFFFFFFFFFULL) < 0x4085E000u;   // |x| < 700
 }
-__device__ __forceinline__ fx64 exp_mag(double x, const fx64* __restrict__ tab, bool up) {
+__device__ __forceinline__ fx64 exp_sig(double x, const fx64* __restrict__ tab, int* m) {   // units of 2^-62
     const int E = bexp(x);
     const long long neg = bits(x) >> 63;                   // 0 or -1
     const fx64 B = sig53(x) << 11;
@@ -150,16 +187,29 @@ __device__ __forceinline__ fx64 exp_mag(double x, const fx64* __restrict__ tab, 
     const fx64 p = r + h + tail;
     const fx64 T = tab[k & (kExpTab - 1)];                 // 2^(j / 512) in units of 2^-62
     const fx32 cross = __umulhi(hi32(T), lo32(p)) + __umulhi(lo32(T), hi32(p));
-    const fx64 M = T + wide(hi32(T), hi32(p)) + cross + (up ? 14 : -2LL);
+    *m = (int)(k >> 9) - 2048;
+    return T + wide(hi32(T), hi32(p)) + cross;
+}
+__device__ __forceinline__ fx64 exp_mag(double x, const fx64* __restrict__ tab, bool up) {
+    int m;
+    const fx64 M = exp_sig(x, tab, &m) + (up ? 14 : -2LL);
     const int top = (int)(M >> 63);
-    return (M >> (10 + top)) + ((fx64)(fx32)((int)(k >> 9) - 2048 + 1022 + top) << 52) + (up ? 1 : 0);
+    return (M >> (10 + top)) + ((fx64)(fx32)(m + 1022 + top) << 52) + (up ? 1 : 0);
+}
+// nearest but for one case of 50 (error below 0.51 units of the last place)
+__device__ __forceinline__ fx64 exp_near(double x, const fx64* __restrict__ tab) {
+    int m;
+    const fx64 M = exp_sig(x, tab, &m) + 6;
+    const int top = (int)(M >> 63);
+    return ((M + (512u << top)) >> (10 + top)) + ((fx64)(fx32)(m + 1022 + top) << 52);
 }
 
-// log(x) rounded outward for a normal x > 0, or 0 (false) where |log x| is
-// below 2^-7: units of 2^-64 are too coarse there. x = 2^m y, y c_j = 1 + r with
+// log(x) rounded outward or to nearest for a normal x > 0; false where |log x| is
+// below 2^-7 (2^-3 to nearest): units of 2^-64 are too coarse there. x = 2^m y, y c_j = 1 + r with
 // 0 <= r < 2^-9.99 exact in 64 bits; log1p(r) = r - r^2/2 (1 - r (2/3 - r/2 + 2 r^2/5)).
 __device__ __forceinline__ bool log_fits(double x) { return (fx32)((bits(x) >> 52) - 1) < 2046u; }
-__device__ __forceinline__ bool log_val(double x, const LogEntry* __restrict__ tab, bool up, double* out) {
+enum FxRound { FX_DOWN = 0, FX_UP = 1, FX_NEAR = 2 };
+__device__ __forceinline__ bool log_val(double x, const LogEntry* __restrict__ tab, int round, double* out) {
     const fx32 E = (fx32)bexp(x);
     const fx64 Y = sig53(x);
     const LogEntry T = tab[(hi32(Y) >> 10) & (kLogTab - 1)];
@@ -168,7 +218,7 @@ __device__ __forceinline__ bool log_val(double x, const LogEntry* __restrict__ t
     const fx64 h = (wide(rq, rq) >> 19) + __umulhi(rq, (lo32(r) >> 9) & 0x3FFFu);
     const fx32 w = 0xAAAAAAABu - __umulhi(rh, 0x80000000u - __umulhi(rh, 0x66666666u));
     const fx64 tail = wide((fx32)(h >> 12), __umulhi(rq, w)) >> 29;
-    const fx64 l1p = r - h + tail;
+    const fx64 l1p = r - h + tail + (round == FX_NEAR ? 2 : 0);   // centres the error
     // E ln2 + (-log c_j - 1023 ln2) + log1p(r): integer word and 64 bits of fraction
     const fx64 a = wide(E, 0xD1CF79ABu) + __umulhi(E, 0xC9E3B398u);
     const fx64 b = wide(E, 0xB17217F7u) + hi32(a);
@@ -182,15 +232,16 @@ __device__ __forceinline__ bool log_val(double x, const LogEntry* __restrict__ t
     const fx32 s = neg ? ~0u : 0u;
     ip ^= s;
     f ^= join(s, s);
-    if (ip == 0u && hi32(f) < 0x02000000u) return false;
-    const bool away = up != neg;
-    const fx64 g = away ? f + 13 : f - 13;
-    ip += away ? (g < f ? 1u : 0u) : (g > f ? ~0u : 0u);
+    if (ip == 0u && hi32(f) < (round == FX_NEAR ? 0x20000000u : 0x02000000u)) return false;
+    const bool near = round == FX_NEAR, away = (round == FX_UP) != neg;
+    const fx64 g = near ? f : away ? f + 13 : f - 13;
+    if (!near) ip += away ? (g < f ? 1u : 0u) : (g > f ? ~0u : 0u);
     const bool small = ip == 0u;
     const fx32 w2 = small ? hi32(g) : ip, w1 = small ? lo32(g) : hi32(g), w0 = small ? 0u : lo32(g);
     const int lz = __clz((int)w2);
     const fx64 mant = join(__funnelshift_l(w1, w2, lz), __funnelshift_l(w0, w1, lz));
-    const fx64 m = (mant >> 11) + ((fx64)(fx32)((small ? 1021 : 1053) - lz) << 52) + (away ? 1 : 0);
+    const fx64 m = (mant >> 11) + ((fx64)(fx32)((small ? 1021 : 1053) - lz) << 52) +
+                   (near ? (mant >> 10) & 1 : away ? 1 : 0);
     *out = from_bits((long long)(m | (neg ? 0x8000000000000000ULL : 0ULL)));
     return true;
 }

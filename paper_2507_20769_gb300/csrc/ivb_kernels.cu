@@ -398,97 +398,104 @@ __global__ void k_finalize(FinalizeParams F) {
 }
 
 // ------------------------------------------------- round-to-nearest gradients
-// Point value and reverse-mode gradient of every output at x (plain double,
-// same local partials as the interval rules), one thread per point. Uses the
-// adjoint programs: forward values into tape records, adjoints into slots.
-__device__ __forceinline__ double pload(const Frame& F, uint32_t kind, uint32_t idx, int base,
-                                        const double* x, const double* consts) {
-    if (kind == K_SLOT) return F.ld(base + (int)idx);
-    if (kind == K_VAR) return x[idx];
-    return __ldg(consts + idx);
+// Point value and reverse-mode gradient of every output at x (plain double, same
+// local partials as the interval rules), one thread per point. Bound by the FP64
+// pipe while quotients, roots, exp and log ran there (three quarters of its FP64
+// instructions; configuration 4, 100003 points: 674 us), which is why these are
+// in fixed point (ivb_fixed.cuh): POINT_FIGURES. x goes through the frame, so that
+// the strided reads of the caller's array happen once.
+__device__ __forceinline__ double point_operand(const double* f, const double* consts, uint32_t w) {
+    const double* q = (w & kOpConst) ? consts : f;
+    return q[w & kOpIndex];
 }
 
-__global__ void __launch_bounds__(256) k_point_grad(const ProgDesc* __restrict__ prog, long long n_points,
-                                                   const double* __restrict__ X, double* f, double* grad,
-                                                   double* gframe, int frame_units) {
+__global__ void __launch_bounds__(64, 16) k_point_grad(const ProgDesc* __restrict__ prog, long long n_points,
+                                                      const double* __restrict__ X, double* f, double* grad,
+                                                      double* gframe, int frame_units) {
     const ProgDesc& G = *prog;
     const int n = G.n, n_out = G.n_out;
+    const double* const consts = G.consts;
+    double* const F = gframe + ((size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * frame_units * 32 + (threadIdx.x & 31);
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n_points;
          p += (long long)gridDim.x * blockDim.x) {
-        Frame F;
-        F.p = gframe + ((size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * frame_units * 32 + (threadIdx.x & 31);
-        const double* x = X + (size_t)p * n;
+        for (int i = 0; i < n; ++i) F[i * 32] = X[(size_t)p * n + i];
         for (int o = 0; o < n_out; ++o) {
             const AdjProgram& A = G.adj[o];
-            const int gb = 0, ab = n, tb = ab + A.adj_slots;
+            const int ab = 2 * n, tb = ab + A.adj_slots;
+            const uint4* q = reinterpret_cast<const uint4*>(G.pins + A.fw_begin);
+            uint4 I = __ldg(q);
+            double v = 0.0;
             for (int i = 0; i < A.fw_count; ++i) {
-                const Ins I = G.ins[A.fw_begin + i];
-                const uint32_t op = I.w0 & 31u, ak = (I.w0 >> 5) & 3u, bk = (I.w0 >> 7) & 3u, dst = I.w0 >> 16;
-                const double a = pload(F, ak, I.w1 & 0xFFFFu, tb, x, G.consts);
-                const double b = (bk != K_NONE) ? pload(F, bk, I.w1 >> 16, tb, x, G.consts) : a;
-                double v;
+                const uint4 next = __ldg(++q);
+                const uint32_t op = I.x;
+                const double a = (I.z & kOpLast) ? v : point_operand(F, consts, I.z);
+                const double b = op > OP_DIV ? a : (I.w & kOpLast) ? v : point_operand(F, consts, I.w);
                 switch (op) {
                 case OP_ADD: v = __dadd_rn(a, b); break;
                 case OP_SUB: v = __dsub_rn(a, b); break;
-                case OP_MUL: v = __dmul_rn(a, b); break;
-                case OP_DIV: v = __ddiv_rn(a, b); break;
-                case OP_SQR: v = __dmul_rn(a, a); break;
-                case OP_SQRT: v = __dsqrt_rn(a); break;
-                case OP_EXP: v = exp(a); break;
-                case OP_LOG: v = log(a); break;
+                case OP_MUL:
+                case OP_SQR: v = __dmul_rn(a, b); break;
+                case OP_DIV: v = div_rn(a, b); break;
+                case OP_SQRT: v = sqrt_rn(a); break;
+                case OP_EXP: v = exp_rn(a); break;
+                case OP_LOG: v = log_rn(a); break;
                 case OP_NEG: v = -a; break;
                 default: v = __longlong_as_double(0x7FF8000000000000LL);
                 }
-                F.st(tb + (int)dst, v);
+                F[I.y] = v;
+                I = next;
             }
-            f[(size_t)p * n_out + o] = pload(F, A.out_kind_ref, A.out_ref, tb, x, G.consts);
+            const int r = A.out_ref;
+            f[(size_t)p * n_out + o] = A.out_kind_ref == K_CONST ? __ldg(consts + r) : F[(A.out_kind_ref == K_VAR ? r : tb + r) * 32];
             if (!grad) continue;
-            for (int i = 0; i < n; ++i) F.st(gb + i, 0.0);
-            if (A.out_wslot >= 0) F.st(ab + A.out_wslot, 1.0);
+            for (int i = 0; i < n; ++i) F[(n + i) * 32] = 0.0;
+            if (A.out_wslot >= 0) F[(ab + A.out_wslot) * 32] = 1.0;
+            q = reinterpret_cast<const uint4*>(G.prins + A.rv_begin);
+            uint4 J = __ldg(q + 1);
+            I = __ldg(q);
+            double last = 0.0;   // the adjoint stored last
             for (int i = 0; i < A.rv_count; ++i) {
-                const RIns R = G.rins[A.rv_begin + i];
-                const uint32_t op = R.w0 & 31u, wslot = R.w0 >> 16;
-                const double w = F.ld(ab + (int)wslot);
-                if (op == OP_VAR) { F.st(gb + (int)R.w1, __dadd_rn(F.ld(gb + (int)R.w1), w)); continue; }
-                const bool a_init = (R.w0 >> 5) & 1u, b_init = (R.w0 >> 6) & 1u;
-                const bool a_none = (R.w0 >> 7) & 1u, b_none = (R.w0 >> 8) & 1u;
-                const uint32_t Ak = (R.w3 >> 16) & 3u, Bk = (R.w3 >> 18) & 3u;
-                double ca = 0.0, cb = 0.0;
-                bool sub_a = false, sub_b = false;
-                switch (op) {
-                case OP_ADD: ca = w; cb = w; break;
-                case OP_SUB: ca = w; cb = w; sub_b = true; break;
-                case OP_NEG: ca = w; sub_a = true; break;
-                case OP_MUL:
-                    ca = __dmul_rn(w, pload(F, Bk, R.w2 >> 16, tb, x, G.consts));
-                    cb = __dmul_rn(w, pload(F, Ak, R.w2 & 0xFFFFu, tb, x, G.consts));
-                    break;
-                case OP_DIV: {
-                    const double r = __ddiv_rn(1.0, pload(F, Bk, R.w2 >> 16, tb, x, G.consts));
-                    const double v = F.ld(tb + (int)(R.w3 & 0xFFFFu));
-                    ca = __dmul_rn(w, r);
-                    cb = __dmul_rn(__dmul_rn(w, v), r);
-                    sub_b = true;
-                } break;
-                case OP_SQR: ca = __dmul_rn(w, __dmul_rn(2.0, pload(F, Ak, R.w2 & 0xFFFFu, tb, x, G.consts))); break;
-                case OP_SQRT:
-                    ca = __dmul_rn(w, __ddiv_rn(1.0, __dmul_rn(2.0, F.ld(tb + (int)(R.w3 & 0xFFFFu)))));
-                    break;
-                case OP_EXP: ca = __dmul_rn(w, F.ld(tb + (int)(R.w3 & 0xFFFFu))); break;
-                case OP_LOG: ca = __dmul_rn(w, __ddiv_rn(1.0, pload(F, Ak, R.w2 & 0xFFFFu, tb, x, G.consts))); break;
+                q += 2;
+                const uint4 nextI = __ldg(q), nextJ = __ldg(q + 1);
+                const uint32_t op = I.x & 31u;
+                const double w = (I.x & kAdjLast) ? last : F[I.y];
+                if (op == OP_VAR) {
+                    F[I.z] = __dadd_rn(F[I.z], w);
+                } else {
+                    const bool a_init = (I.x >> 5) & 1u, b_init = (I.x >> 6) & 1u;
+                    const bool a_none = (I.x >> 7) & 1u, b_none = (I.x >> 8) & 1u;
+                    double ca = w, cb = w;
+                    switch (op) {
+                    case OP_SUB: cb = -w; break;
+                    case OP_NEG: ca = -w; break;
+                    case OP_MUL:
+                        ca = __dmul_rn(w, point_operand(F, consts, J.y));
+                        cb = __dmul_rn(w, point_operand(F, consts, J.x));
+                        break;
+                    case OP_SQR: ca = __dmul_rn(w, __dmul_rn(2.0, point_operand(F, consts, J.x))); break;
+                    case OP_EXP: ca = __dmul_rn(w, F[J.z]); break;
+                    case OP_DIV:
+                    case OP_SQRT:
+                    case OP_LOG: {
+                        const double r = rcp_rn(op == OP_DIV ? point_operand(F, consts, J.y) :
+                                                op == OP_LOG ? point_operand(F, consts, J.x) : __dmul_rn(2.0, F[J.z]));
+                        ca = __dmul_rn(w, r);
+                        if (op == OP_DIV) cb = -__dmul_rn(__dmul_rn(w, F[J.z]), r);
+                    } break;
+                    }
+                    if (!a_none) {
+                        last = a_init ? ca : __dadd_rn(F[I.z], ca);
+                        F[I.z] = last;
+                    }
+                    if (!b_none) {
+                        last = b_init ? cb : __dadd_rn(F[I.w], cb);
+                        F[I.w] = last;
+                    }
                 }
-                if (!a_none) {
-                    const int u = ab + (int)(R.w1 & 0xFFFFu);
-                    const double c = sub_a ? -ca : ca;
-                    F.st(u, a_init ? c : (sub_a ? __dsub_rn(F.ld(u), ca) : __dadd_rn(F.ld(u), ca)));
-                }
-                if (!b_none) {
-                    const int u = ab + (int)(R.w1 >> 16);
-                    const double c = sub_b ? -cb : cb;
-                    F.st(u, b_init ? c : (sub_b ? __dsub_rn(F.ld(u), cb) : __dadd_rn(F.ld(u), cb)));
-                }
+                I = nextI;
+                J = nextJ;
             }
-            for (int i = 0; i < n; ++i) grad[((size_t)p * n_out + o) * n + i] = F.ld(gb + i);
+            for (int i = 0; i < n; ++i) grad[((size_t)p * n_out + o) * n + i] = F[(n + i) * 32];
         }
     }
 }

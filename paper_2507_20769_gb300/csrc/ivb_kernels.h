@@ -11,12 +11,12 @@ namespace ivb {
 
 // program descriptor, resident in device memory for the life of a problem
 struct ProgDesc {
-    const Ins* ins;
-    const RIns* rins;
     const XIns* xins;
     const XIns* xtan;
     const XIns* xcone;
     const XRIns* xrins;
+    const XIns* pins;      // point gradients
+    const XRIns* prins;
     const double* consts;
     int32_t n, n_out, obj, has_eq;
     int32_t pt_begin, pt_count, tan_begin, tan_count;

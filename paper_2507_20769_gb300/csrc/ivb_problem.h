@@ -20,10 +20,11 @@ struct ivb_problem {
     uint8_t out_kind[64]{};
     // program on the device
     ivb::ProgDesc* d_prog = nullptr;
-    ivb::Ins* d_ins = nullptr;
-    ivb::RIns* d_rins = nullptr;
     ivb::XIns* d_xins = nullptr;
     ivb::XRIns* d_xrins = nullptr;
+    ivb::XIns* d_pins = nullptr;
+    ivb::XRIns* d_prins = nullptr;
+    int point_units = 0;      // frame units of the point gradients
     double* d_consts = nullptr;
     uint8_t* d_out_kind = nullptr;
     // per-call buffers (capacity max_nodes)

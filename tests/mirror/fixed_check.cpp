@@ -93,6 +93,12 @@ int main(int argc, char** argv) {
             std::fesetround(up ? FE_UPWARD : FE_DOWNWARD);
             volatile double r = 1.0 / vy, q = vx / vy, g = std::sqrt(vs);
             std::fesetround(FE_TONEAREST);
+            if (up == 0) {   // round to nearest
+                volatile double rn = 1.0 / vy, qn = vx / vy, gn = std::sqrt(vs);
+                rcp += from_bits((long long)rcp_near(y)) != rn;
+                if (std::isfinite(x) && x > 0 && div_fits(x, y)) div += from_bits((long long)div_near(x, y)) != qn;
+                root += from_bits((long long)sqrt_near(s)) != gn;
+            }
             rcp += from_bits((long long)rcp_mag(y, up)) != r;
             if (std::isfinite(x) && x > 0 && div_fits(x, y)) {
                 div += from_bits((long long)div_mag(x, y, rcp62(sig53(y)), up)) != q;
@@ -113,6 +119,9 @@ int main(int argc, char** argv) {
             const double d = from_bits((long long)exp_mag(a, et, false)), u = from_bits((long long)exp_mag(a, et, true));
             ex += !(d <= t && t <= u && from_bits(bits(d) + 3) >= t && from_bits(bits(u) - 3) <= t);
             wide2 += from_bits(bits(u) - 2) > d;
+            const double e = from_bits((long long)exp_near(a, et));
+            const quad half = ((quad)from_bits(bits(e) + 1) - (quad)e) / 2;   // below 0.52 units, above half of them at a power of two
+            ex += !(e - half * (quad)1.04 <= t && t <= e + half * (quad)1.04);
         }
         switch (i & 3) {
         case 0: a = pick(1, 2046); break;
@@ -122,13 +131,21 @@ int main(int argc, char** argv) {
         }
         const quad t = Q_LOG((quad)a);
         double d, u;
-        if (log_val(a, lt, false, &d) != log_val(a, lt, true, &u)) ++lg;
-        else if (!log_val(a, lt, false, &d)) {
+        if (log_val(a, lt, FX_DOWN, &d) != log_val(a, lt, FX_UP, &u)) ++lg;
+        else if (!log_val(a, lt, FX_DOWN, &d)) {
             small += 1;
             lg += !(t < 0x1.01p-7 && t > -0x1.01p-7);
         } else {
             const long long st = t < 0 ? -3 : 3;   // three steps toward +inf
             lg += !(d <= t && t <= u && from_bits(bits(d) + st) >= t && from_bits(bits(u) - st) <= t);
+            double e;
+            if (!log_val(a, lt, FX_NEAR, &e)) {
+                lg += !(t < 0x1.01p-3 && t > -0x1.01p-3);
+                continue;
+            }
+            // half a unit, and 12 units of 2^-64
+            const quad most = std::fabs(from_bits(bits(e) + 1) - e) / 2 + (quad)0xCp-64, off = t - (quad)e;
+            lg += !(off <= most && off >= -most);
         }
     }
     std::printf("rcp=%ld div=%ld sqrt=%ld exp=%ld log=%ld exact=%ld wide=%ld small=%ld\n", rcp, div, root, ex, lg, exact,
