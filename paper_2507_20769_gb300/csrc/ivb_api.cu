@@ -648,6 +648,11 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     CKC(cudaMemcpy(p->d_pins, pins.data(), pins.size() * sizeof(XIns), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(p->d_prins, prins.data(), prins.size() * sizeof(XRIns), cudaMemcpyHostToDevice));
     ProgDesc D{};
+    std::vector<uint32_t> masks;
+    tangent_masks(p->P, ins, masks, D.tan_out_mask);
+    CKC(cudaMalloc(&p->d_tan_mask, masks.size() * sizeof(uint32_t)));
+    CKC(cudaMemcpy(p->d_tan_mask, masks.data(), masks.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    D.tan_mask = reinterpret_cast<const uint2*>(p->d_tan_mask);
     D.pins = p->d_pins;
     D.prins = p->d_prins;
     D.xins = p->d_xins;
@@ -1134,6 +1139,7 @@ extern "C" void ivb_destroy(ivb_problem* p) {
     cudaFree(p->d_prog);
     cudaFree(p->d_xins);
     cudaFree(p->d_xrins);
+    cudaFree(p->d_tan_mask);
     cudaFree(p->d_pins);
     cudaFree(p->d_prins);
     cudaFree(p->d_consts);

@@ -449,4 +449,18 @@ int point_programs(const HostProgram& P, const std::vector<Ins>& ins, const std:
     return units;
 }
 
+void tangent_masks(const HostProgram& P, const std::vector<Ins>& ins, std::vector<uint32_t>& masks, uint32_t out_mask[64]) {
+    masks.assign(2 * (size_t)P.tan_count + 2, 0u);
+    std::vector<uint32_t> slot(P.tan_slots + 1, 0u);   // what the value now in a slot depends on
+    auto of = [&](uint32_t kind, uint32_t idx) { return kind == K_SLOT ? slot[idx] : kind == K_VAR ? 1u << idx : 0u; };
+    for (int i = 0; i < P.tan_count; ++i) {
+        const Ins& I = ins[P.tan_begin + i];
+        const uint32_t a = of((I.w0 >> 5) & 3u, I.w1 & 0xFFFFu), b = of((I.w0 >> 7) & 3u, I.w1 >> 16);
+        masks[2 * i] = a;
+        masks[2 * i + 1] = b;
+        slot[I.w0 >> 16] = a | b;
+    }
+    for (int o = 0; o < P.n_out; ++o) out_mask[o] = of((uint32_t)P.tan_out_kind[o], (uint32_t)P.tan_out_ref[o]);
+}
+
 }  // namespace ivb

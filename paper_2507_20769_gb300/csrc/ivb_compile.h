@@ -30,4 +30,8 @@ void interpreter_programs(const HostProgram& P, const std::vector<Ins>& ins, con
 int point_programs(const HostProgram& P, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
                    std::vector<XIns>& xins, std::vector<XRIns>& xrins);
 
+// variables that the operands of each tangent instruction depend on (bit i: x_i;
+// a at 2k, b at 2k + 1), and each output
+void tangent_masks(const HostProgram& P, const std::vector<Ins>& ins, std::vector<uint32_t>& masks, uint32_t out_mask[64]);
+
 }  // namespace ivb

@@ -13,6 +13,8 @@ namespace ivb {
 struct ProgDesc {
     const XIns* xins;
     const XIns* xtan;
+    const uint2* tan_mask;             // per tangent instruction: variables its operands depend on
+    uint32_t tan_out_mask[64];         // and each output
     const XIns* xcone;
     const XRIns* xrins;
     const XIns* pins;      // point gradients

@@ -22,6 +22,7 @@ struct ivb_problem {
     ivb::ProgDesc* d_prog = nullptr;
     ivb::XIns* d_xins = nullptr;
     ivb::XRIns* d_xrins = nullptr;
+    uint32_t* d_tan_mask = nullptr;
     ivb::XIns* d_pins = nullptr;
     ivb::XRIns* d_prins = nullptr;
     int point_units = 0;      // frame units of the point gradients
