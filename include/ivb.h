@@ -127,7 +127,7 @@ typedef struct {
                                   mode only; for large tapes);
                                   0 (default): tape interpreter; -1: as 1 when
                                   the tape has at most 1024 interval
-                                  operations per subdomain (256 in adjoint
+                                  operations per subdomain (128 in adjoint
                                   mode), else as 3 in adjoint mode and the
                                   interpreter in forward mode, and the
                                   autotuner keeps the interpreter instead
@@ -160,7 +160,8 @@ typedef struct {
                                   warps of a block) share one subdomain, each
                                   running the programs of a group of its
                                   outputs; 0 (default): chosen by the
-                                  autotuner among those compiled            */
+                                  autotuner among those compiled, and more
+                                  of them in calls of few subdomains        */
     int32_t seg_sync;          /* segmented kernel: 1 the warps of a thread
                                   group wait for each other after every chunk
                                   function (they then run the same code and

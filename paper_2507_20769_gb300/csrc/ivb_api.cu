@@ -155,13 +155,18 @@ ivb_status stage_queue(ivb_problem* p, int n_nodes, const double* boxes, const i
     return IVB_OK;
 }
 
+void drop_graphs(ivb_problem* p) {
+    for (cudaGraphExec_t& g : p->gexec)
+        if (g) { cudaGraphExecDestroy(g); g = nullptr; }
+}
+
 ivb_status ensure_frame(ivb_problem* p, int grid, int block, int units) {
     const size_t need = (size_t)grid * block * units * sizeof(double);
     if (need <= p->frame_bytes) return IVB_OK;
     if (p->d_frame) cudaFree(p->d_frame);
     p->d_frame = nullptr;
     p->frame_bytes = 0;
-    if (p->gexec) { cudaGraphExecDestroy(p->gexec); p->gexec = nullptr; }
+    drop_graphs(p);
     CK(cudaMalloc(&p->d_frame, need));
     p->frame_bytes = need;
     return IVB_OK;
@@ -240,6 +245,19 @@ std::vector<int> tpsub_choices(const ivb_problem* p) {
                 v.push_back(t);
     if (p->opt.threads_per_subdomain > 1 && v.size() > 1) v.erase(v.begin());   // a fixed T > 1 excludes 1
     return v;
+}
+
+// Threads per subdomain of one call. A call whose subdomains do not fill the
+// resident threads runs at the latency of its program, so the outputs of a
+// subdomain are shared among as many threads as stay resident, unless an option
+// fixes their number or the grabs (1024 subdomains of configuration 2, 4 outputs: 147 us with 1
+// thread, 94 with 2, 76 with 4).
+int call_tpsub(const ivb_problem* p, long long total, long long threads) {
+    if (!reduce_jit(p) || p->opt.threads_per_subdomain != 0 || p->opt.tile > 0 || p->jit.ilp != 1) return p->tpsub;
+    int best = p->tpsub;
+    for (int t : {2, 4})
+        if (t > best && p->jit.kern_t[tpsub_index(t)] && p->block % (32 * t) == 0 && total * t <= threads) best = t;
+    return best;
 }
 
 // chunk synchronisation choices: the segmented kernels come with and without;
@@ -368,7 +386,7 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
     p->tune_worst_ms = worst;
     p->tuned = true;
     p->cfg_ready = true;
-    if (p->gexec) { cudaGraphExecDestroy(p->gexec); p->gexec = nullptr; }
+    drop_graphs(p);
     return IVB_OK;
 }
 
@@ -826,26 +844,29 @@ ivb_status bound_nodes_impl(ivb_problem* p, int32_t n_nodes, const double* boxes
         const int grid = p->sm_count * p->bps;
         if (reduce_units(p) > 0) st = ensure_frame(p, grid, p->block, reduce_units(p));
         if (st) return st;
+        const int tpsub = call_tpsub(p, total, (long long)grid * p->block);
+        const int tile = tpsub == p->tpsub ? p->tile : pass_size(p, p->block, tpsub);
         if (p->opt.use_graph) {
-            if (!p->gexec) {
+            cudaGraphExec_t& gexec = p->gexec[tpsub_index(tpsub)];
+            if (!gexec) {
                 cudaGraph_t g = nullptr;
                 CK(cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal));
-                st = enqueue_bound(p, grid, p->block, p->tile, p->frame_smem, p->max_nodes, p->cap_stream, p->tpsub,
+                st = enqueue_bound(p, grid, p->block, tile, p->frame_smem, p->max_nodes, p->cap_stream, tpsub,
                                    p->chunk_sync);
                 cudaGraph_t gg = nullptr;
                 cudaError_t ce = cudaStreamEndCapture(p->cap_stream, &gg);
                 if (st) { if (gg) cudaGraphDestroy(gg); return st; }
                 if (ce != cudaSuccess) return cuda_fail(p, ce, "cudaStreamEndCapture");
                 g = gg;
-                ce = cudaGraphInstantiate(&p->gexec, g, 0);
+                ce = cudaGraphInstantiate(&gexec, g, 0);
                 cudaGraphDestroy(g);
-                if (ce != cudaSuccess) { p->gexec = nullptr; return cuda_fail(p, ce, "cudaGraphInstantiate"); }
+                if (ce != cudaSuccess) { gexec = nullptr; return cuda_fail(p, ce, "cudaGraphInstantiate"); }
                 p->launches -= 3;   // captured, not launched
             }
-            CK(cudaGraphLaunch(p->gexec, s));
+            CK(cudaGraphLaunch(gexec, s));
             p->launches += 3;
         } else {
-            st = enqueue_bound(p, grid, p->block, p->tile, p->frame_smem, p->max_nodes, s, p->tpsub, p->chunk_sync);
+            st = enqueue_bound(p, grid, p->block, tile, p->frame_smem, p->max_nodes, s, tpsub, p->chunk_sync);
             if (st) return st;
         }
     }
@@ -1133,7 +1154,7 @@ extern "C" const char* ivb_last_error(const ivb_problem* p) {
 
 extern "C" void ivb_destroy(ivb_problem* p) {
     if (!p) return;
-    if (p->gexec) cudaGraphExecDestroy(p->gexec);
+    drop_graphs(p);
     if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
     if (p->queue_free) { cudaEventSynchronize(p->queue_free); cudaEventDestroy(p->queue_free); }
     cudaFree(p->d_prog);

@@ -24,9 +24,10 @@ namespace ivb {
 // compile time grows to tens of seconds and the interpreter was within 5 % on
 // the configurations measured). In adjoint mode the segmented kernel takes
 // over from kSegMinOps on: with 32 warps per SM it is ahead at 620 operations
-// (configuration 2, 16 nodes x 16^4: 2.4 to 2.6 ms against 2.75) and compiles in a
-// tenth of the time; below, there is little to cut.
-constexpr int kJitBlockMax = 256, kJitMinBlocks = 2, kJitAutoMaxOps = 1024, kSegMinOps = 256;
+// (configuration 2, 16 nodes x 16^4: 2.06 ms against 2.75) and compiles in a
+// tenth of the time; at 231 operations and two outputs a small call takes 52 us
+// against 65 (call_tpsub); below, there is little to cut.
+constexpr int kJitBlockMax = 256, kJitMinBlocks = 2, kJitAutoMaxOps = 1024, kSegMinOps = 128;
 // chunks from which a segmented kernel keeps its warps on one chunk (below, the
 // autotuner times both). Warps that drift apart stream through the code
 // separately, and a sample of uniform subdomains does not show it: 306 chunks 56

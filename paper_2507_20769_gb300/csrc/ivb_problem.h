@@ -54,7 +54,7 @@ struct ivb_problem {
     int tune_candidates = 0;  // launch configurations the autotuner timed
     float tune_best_ms = 0.f, tune_worst_ms = 0.f;
     // graph of the batched call
-    cudaGraphExec_t gexec = nullptr;
+    cudaGraphExec_t gexec[3] = {nullptr, nullptr, nullptr};   // by threads per subdomain (tpsub_index)
     cudaStream_t cap_stream = nullptr;
     // point gradients
     double* d_pframe = nullptr;
