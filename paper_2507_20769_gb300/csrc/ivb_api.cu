@@ -184,6 +184,7 @@ KParams make_params(ivb_problem* p, int frame_smem) {
     K.frame_units = reduce_units(p);
     K.keys = p->d_keys;
     K.form = p->opt.form;
+    K.groups = 1;
     return K;
 }
 
@@ -192,8 +193,9 @@ size_t smem_bytes(const ivb_problem* p, int block, int frame_smem) {
 }
 
 // the reduce-mode bounding kernel: tape-specialised when compiled, else the interpreter
-cudaError_t launch_reduce(ivb_problem* p, const KParams& K, int grid, int block, int frame_smem, cudaStream_t s,
+cudaError_t launch_reduce(ivb_problem* p, KParams K, int grid, int block, int frame_smem, cudaStream_t s,
                           int tpsub, bool sync) {
+    K.groups = tpsub;
     if (reduce_jit(p)) return jit_launch(p->jit, K, grid, block, s, tpsub, sync);
     return launch_bound(kernel_mode(p, false), K, grid, block, smem_bytes(p, block, frame_smem), s);
 }
@@ -251,12 +253,16 @@ std::vector<int> tpsub_choices(const ivb_problem* p) {
 // resident threads runs at the latency of its program, so the outputs of a
 // subdomain are shared among as many threads as stay resident, unless an option
 // fixes their number or the grabs (1024 subdomains of configuration 2, 4 outputs: 147 us with 1
-// thread, 94 with 2, 76 with 4).
+// thread, 94 with 2, 76 with 4; the interpreter shares them among warp groups:
+// 297 us with one group, 103 with 4).
 int call_tpsub(const ivb_problem* p, long long total, long long threads) {
-    if (!reduce_jit(p) || p->opt.threads_per_subdomain != 0 || p->opt.tile > 0 || p->jit.ilp != 1) return p->tpsub;
+    if (p->opt.threads_per_subdomain != 0 || p->opt.tile > 0 || (reduce_jit(p) && p->jit.ilp != 1)) return p->tpsub;
     int best = p->tpsub;
-    for (int t : {2, 4})
-        if (t > best && p->jit.kern_t[tpsub_index(t)] && p->block % (32 * t) == 0 && total * t <= threads) best = t;
+    for (int t : {2, 4}) {
+        const bool can = reduce_jit(p) ? p->jit.kern_t[tpsub_index(t)] != nullptr
+                                       : p->opt.grad_mode == IVB_GRAD_ADJOINT && t <= p->n_out;
+        if (t > best && can && p->block % (32 * t) == 0 && total * t <= threads) best = t;
+    }
     return best;
 }
 

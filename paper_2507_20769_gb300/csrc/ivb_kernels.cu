@@ -227,8 +227,11 @@ __global__ void __launch_bounds__(512, 2) k_bound(const KParams P) {
     C.consts = G.consts;
     C.x_base = L.x_base;
 
-    const int groups = MODE == KM_ADJ_STORE ? P.groups : 1;
-    const int per = (int)blockDim.x / groups, first_o = MODE == KM_ADJ_STORE ? (int)threadIdx.x / per : 0;
+    // adjoint modes: the outputs of a subdomain shared among warp groups (KParams::groups)
+    constexpr bool kAdj = MODE == KM_ADJ_STORE || MODE == KM_ADJ_REDUCE;
+    const int groups = kAdj ? P.groups : 1;
+    const int per = (int)blockDim.x / groups, first_o = kAdj ? (int)threadIdx.x / per : 0;
+    __shared__ unsigned char s_fl[512];
     tile_loop_per(P, per, [&](const Sub& s) {
         const long long g = s.g;
         const bool valid = s.valid;
@@ -254,8 +257,8 @@ __global__ void __launch_bounds__(512, 2) k_bound(const KParams P) {
         // With the natural interval extension alone (form 1) a reduce launch needs no
         // gradients: only the value sweep over X_k.
         const bool nie_only = (MODE == KM_FWD_REDUCE || MODE == KM_ADJ_REDUCE) && P.form == 1;
-        bool cert_infeasible = false;
-        double obj_lo = from_bits(0x7FF0000000000000LL);
+        unsigned fl = 0;   // bit 0: an output proves the subdomain infeasible; bit 1: its centre is not certified feasible
+        double obj_lo = from_bits(0x7FF0000000000000LL), obj_c = obj_lo;
         if (MODE == KM_FWD_REDUCE || MODE == KM_FWD_STORE) {
             if (valid) {
                 if (nie_only) run_values(G.xtan, G.tan_count, C);
@@ -264,8 +267,20 @@ __global__ void __launch_bounds__(512, 2) k_bound(const KParams P) {
         }
         for (int o = first_o; o < n_out; o += groups) {
             iv F = zero(), Fc = zero();
+            if (valid) {
+                if (groups > 1) {   // f(c) of this output alone
+                    const AdjProgram& A = G.adj[o];
+                    const int tb = L.phase_base + 2 * n + 2 * A.adj_slots;
+                    run_values(G.xcone + A.fw_begin, A.fw_count, C);
+                    const double c = A.out_kind_ref == K_VAR ? C.F.ld(L.c_base + A.out_ref) : 0.0;
+                    Fc = A.out_kind_ref == K_VAR ? mk(c, c) : load_val(C, A.out_kind_ref, A.out_ref, tb, 2);
+                } else {
+                    Fc = C.F.get(L.fc_base + 2 * o);
+                }
+                if (G.out_kind[o] == OUT_INEQ && !le0(Fc.hi)) fl |= 2u;
+                if (o == G.obj) obj_c = Fc.hi;
+            }
             if (valid && nie_only) {
-                Fc = C.F.get(L.fc_base + 2 * o);
                 iv nie;
                 if (MODE == KM_FWD_REDUCE) {
                     nie = load_val(C, G.tan_out_kind[o], G.tan_out_ref[o], L.phase_base, L.tan_rec);
@@ -276,18 +291,9 @@ __global__ void __launch_bounds__(512, 2) k_bound(const KParams P) {
                     nie = load_val(C, A.out_kind_ref, A.out_ref, tb, 2);
                 }
                 F = final_form(1, nie, nie);
-                if (excludes_feasible(G.out_kind[o], F)) cert_infeasible = true;
+                if (excludes_feasible(G.out_kind[o], F)) fl |= 1u;
                 if (o == G.obj) obj_lo = F.lo;
             } else if (valid) {
-                if (groups > 1) {   // f(c) of this output alone
-                    const AdjProgram& A = G.adj[o];
-                    const int tb = L.phase_base + 2 * n + 2 * A.adj_slots;
-                    run_values(G.xcone + A.fw_begin, A.fw_count, C);
-                    const double c = A.out_kind_ref == K_VAR ? C.F.ld(L.c_base + A.out_ref) : 0.0;
-                    Fc = A.out_kind_ref == K_VAR ? mk(c, c) : load_val(C, A.out_kind_ref, A.out_ref, tb, 2);
-                } else {
-                    Fc = C.F.get(L.fc_base + 2 * o);
-                }
                 iv nie;
                 int gunit, gstride;  // gradient of this output: unit of G_0 and stride (0: constant/variable)
                 uint32_t dirs = ~0u;  // directions it depends on
@@ -324,7 +330,7 @@ __global__ void __launch_bounds__(512, 2) k_bound(const KParams P) {
                     }
                 }
                 F = final_form(P.form, mvf, nie);
-                if (excludes_feasible(G.out_kind[o], F)) cert_infeasible = true;
+                if (excludes_feasible(G.out_kind[o], F)) fl |= 1u;
                 if (o == G.obj) obj_lo = F.lo;
             }
             if (MODE == KM_FWD_STORE || MODE == KM_ADJ_STORE) {
@@ -343,15 +349,18 @@ __global__ void __launch_bounds__(512, 2) k_bound(const KParams P) {
             }
         }
         if (MODE == KM_FWD_REDUCE || MODE == KM_ADJ_REDUCE) {
-            double ub = from_bits(0x7FF0000000000000LL);
-            if (valid) {
-                bool feas = !G.has_eq;
-                for (int o = 0; o < n_out; ++o)
-                    if (G.out_kind[o] == OUT_INEQ && !le0(C.F.ld(L.fc_base + 2 * o + 1))) feas = false;
-                if (feas) ub = C.F.ld(L.fc_base + 2 * G.obj + 1);
-                if (cert_infeasible) obj_lo = from_bits(0x7FF0000000000000LL);
+            if (groups > 1) {   // the objective's group needs every output's tests
+                s_fl[threadIdx.x] = (unsigned char)fl;
+                __syncthreads();
+                for (int h = 0; h < groups; ++h) fl |= s_fl[h * per + (int)threadIdx.x % per];
+                __syncthreads();
             }
-            reduce_extras(P, s, n_out, ub, obj_lo);
+            if (G.obj % groups == first_o) {
+                double ub = from_bits(0x7FF0000000000000LL);
+                if (valid && !G.has_eq && !(fl & 2u)) ub = obj_c;
+                if (fl & 1u) obj_lo = from_bits(0x7FF0000000000000LL);
+                reduce_extras(P, s, n_out, ub, obj_lo);
+            }
         }
     });
 }

@@ -51,7 +51,7 @@ struct KParams {
     double* outG;
     long long store_first_g;   // first global index of the call (0 in the reduce modes)
     int32_t form;          // 0 MVF, 1 NIE, 2 MVF meet NIE
-    int32_t groups;        // adjoint store mode: warp groups of a block that share the outputs of its subdomains
+    int32_t groups;        // interpreter, adjoint modes: warp groups of a block that share its subdomains' outputs
 };
 
 }  // namespace ivb

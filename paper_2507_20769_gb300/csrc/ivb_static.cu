@@ -179,6 +179,7 @@ extern "C" ivb_status ivb_bound_nodes_noalloc(ivb_problem* p, int32_t n_nodes, c
     K.frame_units = fu;
     K.keys = keys;
     K.form = p->opt.form;
+    K.groups = 1;
     CKN(launch_bound(mode, K, p->sm_count * bps, block, smem, s));
     FinalizeParams F{};
     F.keys = keys;
