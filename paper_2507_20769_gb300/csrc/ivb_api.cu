@@ -285,7 +285,7 @@ std::vector<bool> sync_choices(const ivb_problem* p) {
 // times larger grabs (4 and 16 passes per grab) for the best of stage 1.
 ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
     std::vector<TuneCand> cands;
-    const int blocks[] = {1024, 512, 64, 128, 256};   // largest: segmented kernels 1024, interpreter 512
+    const int blocks[] = {1024, 512, 256, 128, 64};   // largest: segmented kernels 1024, interpreter 512
     const int bpss[] = {1, 2, 3, 4, 6, 8};
     int max_threads = 0;
     // with the library's choice of kernel, the interpreter competes with the
@@ -326,7 +326,7 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
     CK(cudaEventCreate(&ew));
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    float best = 1e30f, worst = 0.f;
+    float best = 1e30f, worst = 0.f, last_ms = 0.f;
     TuneCand bc = cands[0];
     ivb_status st = IVB_OK;
     int timed = 0;
@@ -354,15 +354,30 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
             CK(cudaEventElapsedTime(&ms, e0, e1));
         }
         ++timed;
+        last_ms = ms;
         worst = std::max(worst, ms);
         if (ms < best) { best = ms; bc = c; }
         return IVB_OK;
     };
-    for (const TuneCand& c : cands) {
+    // Blocks come largest first. When the best launch of one block size takes over
+    // twice the best time so far, smaller blocks of the same kernel are left out:
+    // their warps share even less code (configuration 5: 68 launches in 16 s, now 47 in
+    // 4 s).
+    float size_ms = 1e30f;      // best time of the block size being timed
+    bool hopeless = false;
+    for (size_t i = 0; i < cands.size() && !st; ++i) {
+        const TuneCand& c = cands[i];
+        const bool same = i > 0 && cands[i - 1].interp == c.interp && cands[i - 1].sync == c.sync && cands[i - 1].tpsub == c.tpsub;
+        if (!same) hopeless = false;
+        else if (cands[i - 1].block != c.block) hopeless = hopeless || size_ms > 2.f * best;
+        if (!same || cands[i - 1].block != c.block) size_ms = 1e30f;
+        if (hopeless) continue;
         st = time_one(c);
-        if (st) break;
+        size_ms = std::min(size_ms, last_ms);
     }
-    if (!st && p->opt.tile <= 0) {
+    // larger grabs: not for segmented kernels, whose passes are long and dealt out
+    // evenly (a grab of four passes that fits the sample leaves others unbalanced)
+    if (!st && p->opt.tile <= 0 && (bc.interp || p->jit.state_units == 0)) {
         const TuneCand base = bc;
         for (int mult : {4, 16}) {
             TuneCand c = base;
