@@ -416,8 +416,10 @@ __global__ void k_finalize(FinalizeParams F) {
 // local partials as the interval rules), one thread per point. Bound by the FP64
 // pipe while quotients, roots, exp and log ran there (three quarters of its FP64
 // instructions; configuration 4, 100003 points: 674 us), which is why these are
-// in fixed point (ivb_fixed.cuh): POINT_FIGURES. x goes through the frame, so that
-// the strided reads of the caller's array happen once.
+// in fixed point (ivb_fixed.cuh): 321 us now, and 684 -> 329 us for value and
+// gradient through autograd. Now bound by latency: 44 k instructions per warp of
+// points, waiting on frame loads and long chains. x goes through the frame, so
+// that the strided reads of the caller's array happen once.
 __device__ __forceinline__ double point_operand(const double* f, const double* consts, uint32_t w) {
     const double* q = (w & kOpConst) ? consts : f;
     return q[w & kOpIndex];
