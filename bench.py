@@ -358,9 +358,12 @@ def roofline_block(p, subs_step, step_s, clk, dev, probes=False):
     decode) times the subdomains of a step, over the step time (the bounding
     kernel is > 99.9 % of a step: profiles/ has the launch list). `peak` is the
     FP64 pipe from unit counts and the SM clock sampled during the steps:
-    2 FP64 lanes per clock per SM x SMs x clock. Beside it, the issue-slot view
-    (`pipe_busy_frac`): each category priced in DFMA issue slots at the
-    measured rates of the primitives the kernel runs."""
+    2 FP64 lanes per clock per SM x SMs x clock. Quotients, reciprocals, roots,
+    exp and log are endpoint operations too but run in fixed point on the integer
+    pipes, as do products by powers of two, so `achieved` can pass the FP64
+    pipe's peak. Beside it, the issue-slot view of that pipe (`pipe_busy_frac`):
+    sums, products and decode at one DFMA issue slot each (products by powers
+    of two counted as if they were there)."""
     import torch
     from paper_2507_20769_gb300 import ivb
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
@@ -385,10 +388,8 @@ def roofline_block(p, subs_step, step_s, clk, dev, probes=False):
         for k, extra in (("own_log", "dadd"), ("own_sqrt", "dmul")):
             # these probes carry one extra round-to-nearest add / multiply per operation
             rates[k] = 1.0 / max(1.0 / rates[k] - 1.0 / rates[extra], 1e-30)
-        cost = {"addsub": probe / rates["dadd"], "mul": probe / rates["dmul"], "div": probe / rates["own_div"],
-                "rcp": probe / rates["own_rcp"], "sqrt": probe / rates["own_sqrt"], "exp": probe / rates["own_exp"],
-                "log": probe / rates["own_log"], "rn": probe / rates["dadd"]}
-        slots = sum(counts[k] * cost[k] for k in counts)
+        cost = {"addsub": probe / rates["dadd"], "mul": probe / rates["dmul"], "rn": probe / rates["dadd"]}
+        slots = sum(counts[k] * cost[k] for k in cost)
         rf["pipe_busy_frac"] = slots * subs_step / step_s / peak
         rf["issue_slot_view"] = {"dfma_slots_per_subdomain": slots, "measured_dfma_probe_glanes": probe / 1e9,
                                  "frac_of_measured_probe": slots * subs_step / step_s / probe,
