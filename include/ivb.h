@@ -161,7 +161,10 @@ typedef struct {
                                   running the programs of a group of its
                                   outputs; 0 (default): chosen by the
                                   autotuner among those compiled, and more
-                                  of them in calls of few subdomains        */
+                                  of them in calls of few subdomains. Runs
+                                  with 1 where block_threads is not a
+                                  multiple of 32 times the number (each group
+                                  is whole warps)                           */
     int32_t seg_sync;          /* segmented kernel: 1 the warps of a thread
                                   group wait for each other after every chunk
                                   function (they then run the same code and

@@ -20,7 +20,7 @@ SOURCES = ["ivb_kernels.cu", "ivb_api.cu", "ivb_probe.cu", "ivb_static.cu", "ivb
            "ivb_jit.cpp", "ivb_jit_seg.cpp", "ivb_host.cpp"]
 HEADERS = ["ivb_internal.h", "ivb_iv.cuh", "ivb_fixed.cuh", "ivb_fp64x.cuh", "ivb_emu.cuh", "ivb_kparams.h",
            "ivb_bound_common.cuh", "ivb_kernels.h",
-           "ivb_problem.h", "ivb_jit.h", "ivb_host.h", "ivb_compile.h"]
+           "ivb_problem.h", "ivb_launch.h", "ivb_jit.h", "ivb_host.h", "ivb_compile.h"]
 # device headers the tape-specialised kernels are compiled against at run time (NVRTC)
 JIT_HEADERS = ["ivb_bound_common.cuh", "ivb_internal.h", "ivb_iv.cuh", "ivb_fixed.cuh", "ivb_fp64x.cuh", "ivb_emu.cuh",
                "ivb_kparams.h"]

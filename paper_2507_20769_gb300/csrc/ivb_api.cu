@@ -16,6 +16,7 @@
 #include "ivb_compile.h"
 #include "ivb_internal.h"
 #include "ivb_kernels.h"
+#include "ivb_launch.h"
 #include "ivb_problem.h"
 
 
@@ -261,7 +262,7 @@ int call_tpsub(const ivb_problem* p, long long total, long long threads) {
     for (int t : {2, 4}) {
         const bool can = reduce_jit(p) ? p->jit.kern_t[tpsub_index(t)] != nullptr
                                        : p->opt.grad_mode == IVB_GRAD_ADJOINT && t <= p->n_out;
-        if (t > best && can && p->block % (32 * t) == 0 && total * t <= threads) best = t;
+        if (t > best && can && groups_fit(p->block, t) && total * t <= threads) best = t;
     }
     return best;
 }
@@ -300,7 +301,7 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
         for (int b : blocks)
             for (int k : bpss) {
                 const int warps = b * k / 32;
-                if (warps < 4 || warps > 32 || b < 32 * t) continue;
+                if (warps < 4 || warps > 32 || !groups_fit(b, t)) continue;
                 if (b > (reduce_jit(p) ? (p->jit.state_units > 0 ? p->jit.block_max : 256) : 512)) continue;
                 for (int sm = 0; sm < 2; ++sm) {
                     const size_t bytes = smem_bytes(p, b, sm);
@@ -427,8 +428,7 @@ ivb_status default_tuning(ivb_problem* p) {
     else if (p->opt.frame_in_shared == 1) p->frame_smem = 1;
     else if (p->opt.frame_in_shared == 0) p->frame_smem = 0;
     else p->frame_smem = (bytes + 1024 <= (size_t)p->smem_optin && bytes * p->bps <= 220 * 1024) ? 1 : 0;
-    p->tpsub = tpsub_choices(p).front();
-    if (p->block < 32 * p->tpsub) p->tpsub = 1;
+    p->tpsub = block_tpsub(p->block, tpsub_choices(p).front());
     p->chunk_sync = sync_choices(p).front();
     const int occ = reduce_occupancy(p, p->block, p->frame_smem, p->tpsub, p->chunk_sync);
     if (occ < 1) return fail(p, IVB_ENOTSUP, "launch configuration does not fit on an SM");
@@ -943,7 +943,7 @@ extern "C" ivb_status ivb_enclose(ivb_problem* p, const double* box, const int32
     // subdomains of configuration 3, 6 outputs: 1.38 -> 1.03 ms)
     K.groups = 1;
     if (p->opt.grad_mode == IVB_GRAD_ADJOINT)
-        while (2 * K.groups <= std::min(8, n_out) && block % (64 * K.groups) == 0 &&
+        while (2 * K.groups <= std::min(8, n_out) && groups_fit(block, 2 * K.groups) &&
                2 * K.groups * count <= (long long)grid * block)
             K.groups *= 2;
     K.tile = block / K.groups;

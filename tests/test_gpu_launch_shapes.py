@@ -1,0 +1,53 @@
+"""Launch shapes fixed by options: the shape that runs is the documented one, and
+the bounds are the interpreter's bits at every one of them."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2507_20769_gb300 import build as B  # noqa: E402
+
+B.build()
+from paper_2507_20769_gb300 import ivb  # noqa: E402
+from paper_2507_20769_gb300 import workloads as W  # noqa: E402
+
+KEYS = ("lb", "ub", "minlo", "maxhi", "infeasible")
+
+
+def tape():
+    return W.random_problem(2, 60, 3, W.OPS_ALL, [[-2, 2]] * 2, 51, "launch shapes")
+
+
+def bounds(p, total=7001):
+    boxes = np.array([[[-2.0, 0.5], [-1.0, 2.0]], [[0.5, 2.0], [-2.0, 0.25]]])
+    splits = np.array([[total // 3, 1], [total - total // 3, 1]], np.int32)
+    return p.bound_nodes_ex(boxes, splits, want_hull=True)
+
+
+def assert_same(r, ref, what):
+    for k in KEYS:
+        assert np.array_equal(r[k].view(np.uint8), ref[k].view(np.uint8)), (what, k)
+
+
+@pytest.fixture(scope="module")
+def reference():
+    with ivb.Problem(tape(), specialize=0, autotune=0, threads_per_subdomain=1) as p:
+        return bounds(p)
+
+
+@pytest.mark.parametrize("sync", [0, 1])
+@pytest.mark.parametrize("block,asked,runs", [(96, 2, 1), (96, 4, 1), (160, 2, 1), (192, 2, 2), (192, 4, 1), (32, 2, 1),
+                                              (64, 2, 2), (128, 4, 4)])
+def test_threads_per_subdomain_only_in_whole_warps(reference, block, asked, runs, sync):
+    with ivb.Problem(tape(), specialize=3, seg_chunk=24, block_threads=block, threads_per_subdomain=asked,
+                     seg_sync=sync) as p:
+        r = bounds(p)
+        tun = p.get_tuning()
+    assert (tun["block_threads"], tun["threads_per_subdomain"]) == (block, runs)
+    assert_same(r, reference, (block, asked))
