@@ -930,10 +930,13 @@ extern "C" ivb_status ivb_enclose(ivb_problem* p, const double* box, const int32
     if (out_G && !dG) CK(cudaMallocAsync(&tG, gb, s));
     const unsigned long long first_u = (unsigned long long)first;
     CK(cudaMemcpyAsync(p->d_counter, &first_u, sizeof(first_u), cudaMemcpyHostToDevice, s));
-    // the store modes run the interpreter: its own shape when the reduce launches use another kernel
+    // the store modes run the interpreter: in the shape of the reduce launches where these run it too,
+    // else in the options' or its own
     const bool own = !reduce_jit(p);
-    const int block = own ? p->block : 256, bps = own ? p->bps : 4, fs = own ? p->frame_smem : 0;
-    const int grid = p->sm_count * bps;   // the range is dealt out evenly
+    const int block = own ? p->block : p->opt.block_threads > 0 ? p->opt.block_threads : 256;
+    const int bps = own ? p->bps : p->opt.blocks_per_sm > 0 ? p->opt.blocks_per_sm : 4;
+    const int fs = own ? p->frame_smem : 0;
+    const int resident = p->sm_count * bps, grid = range_blocks(count, resident);   // dealt out evenly
     st = ensure_frame(p, grid, block, frame_units(p));
     if (st) return st;
     KParams K = make_params(p, fs);
@@ -944,7 +947,7 @@ extern "C" ivb_status ivb_enclose(ivb_problem* p, const double* box, const int32
     K.groups = 1;
     if (p->opt.grad_mode == IVB_GRAD_ADJOINT)
         while (2 * K.groups <= std::min(8, n_out) && groups_fit(block, 2 * K.groups) &&
-               2 * K.groups * count <= (long long)grid * block)
+               2 * K.groups * count <= (long long)resident * block)
             K.groups *= 2;
     K.tile = block / K.groups;
     K.outF = dF ? out_F : tF;

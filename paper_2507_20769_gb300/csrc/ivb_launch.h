@@ -13,4 +13,11 @@ inline bool groups_fit(int block, int groups) { return groups >= 1 && block % (3
 // where the block cannot be dealt out to that many groups
 inline int block_tpsub(int block, int wanted) { return groups_fit(block, wanted) ? wanted : 1; }
 
+// Blocks of a launch over `count` subdomains, of `resident` at most: a block takes a
+// warp of subdomains at least (even_tile), further blocks would only hold frames.
+inline int range_blocks(long long count, int resident) {
+    const long long warps = (count + 31) / 32;
+    return warps < resident ? (int)warps : resident;
+}
+
 }  // namespace ivb

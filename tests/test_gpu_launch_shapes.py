@@ -51,3 +51,28 @@ def test_threads_per_subdomain_only_in_whole_warps(reference, block, asked, runs
         tun = p.get_tuning()
     assert (tun["block_threads"], tun["threads_per_subdomain"]) == (block, runs)
     assert_same(r, reference, (block, asked))
+
+
+def used():
+    torch.cuda.synchronize()
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+
+
+@pytest.mark.parametrize("specialize", [0, 3])
+def test_stored_range_holds_frames_of_the_blocks_that_work(specialize):
+    """a long tape (some 6 KB of frame per thread): one subdomain takes a block's frames, and a
+    shape fixed by options bounds those of a range that fills the device; the same bits either way"""
+    wl = W.config_workload(4)
+    box, splits = wl.tape.root_box, np.asarray(wl.splits, np.int32)
+    out = []
+    for opts, ranges in ((dict(), ((77, 1),)), (dict(block_threads=32, blocks_per_sm=1), ((77, 1), (70, 40_000)))):
+        with ivb.Problem(wl.tape, specialize=specialize, autotune=0, **opts) as p:
+            warm = used()
+            for first, count in ranges:
+                out.append(p.enclose(box, splits, first=first, count=count, want_fc=True, want_g=True))
+            assert used() - warm < 128 << 20
+    for k in range(3):
+        a, b, c = (np.asarray(o[k]) for o in out)
+        assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
+        assert np.array_equal(a.view(np.uint8), np.ascontiguousarray(c[7:8]).view(np.uint8))

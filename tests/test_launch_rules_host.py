@@ -37,3 +37,11 @@ def test_groups_of_a_block_are_whole_warps(rows):
         assert block % t == 0 and (block // t) % 32 == 0, (block, wanted, t)
         assert t == (wanted if block % (32 * wanted) == 0 else 1), (block, wanted, t)
     assert [96, 2, 1] in got and [192, 2, 2] in got and [192, 4, 1] in got
+
+
+def test_blocks_of_a_range_all_get_work(rows):
+    """as many blocks as there are warps of subdomains, of the resident ones"""
+    counts = (1, 31, 32, 33, 64, 65, 19455, 19456, 19457, 50003, 1 << 24)
+    got = rows("for (long long c : {%s}) std::printf(\"%%lld %%d\\n\", c, range_blocks(c, 608));"
+               % ", ".join(f"{c}LL" for c in counts))
+    assert got == [[c, min(608, -(-c // 32))] for c in counts]
