@@ -161,15 +161,44 @@ void drop_graphs(ivb_problem* p) {
         if (g) { cudaGraphExecDestroy(g); g = nullptr; }
 }
 
-ivb_status ensure_frame(ivb_problem* p, int grid, int block, int units) {
-    const size_t need = (size_t)grid * block * units * sizeof(double);
-    if (need <= p->frame_bytes) return IVB_OK;
+void free_frame(ivb_problem* p) {
     if (p->d_frame) cudaFree(p->d_frame);
     p->d_frame = nullptr;
     p->frame_bytes = 0;
     drop_graphs(p);
-    CK(cudaMalloc(&p->d_frame, need));
+}
+
+// frames of `units` for a launch of exactly `grid` blocks
+ivb_status ensure_frame(ivb_problem* p, int grid, int block, int units) {
+    const size_t need = (size_t)grid * block * units * sizeof(double);
+    if (need <= p->frame_bytes) return IVB_OK;
+    free_frame(p);
+    const cudaError_t e = cudaMalloc(&p->d_frame, need);
+    if (e != cudaSuccess) {
+        cudaGetLastError();   // the launches that follow check for it
+        p->d_frame = nullptr;
+        return cuda_fail(p, e, "frames");
+    }
     p->frame_bytes = need;
+    return IVB_OK;
+}
+
+// frames for a launch of at most *grid blocks; *grid becomes the number that the memory holds
+ivb_status fit_frame(ivb_problem* p, int* grid, int block, int units) {
+    const size_t per = (size_t)block * units * sizeof(double);
+    if (per == 0) return IVB_OK;
+    if ((size_t)*grid * per > p->frame_most) *grid = std::max(1, (int)(p->frame_most / per));
+    ivb_status st = IVB_OK;
+    const int got = blocks_that_fit(*grid, [&](int g) {
+        st = ensure_frame(p, g, block, units);
+        return st != IVB_ENOMEM;
+    });
+    if (st) return st;
+    if (got < *grid) {
+        p->frame_most = p->frame_bytes;   // not tried again on every call
+        p->err.clear();
+    }
+    *grid = got;
     return IVB_OK;
 }
 
@@ -276,12 +305,14 @@ std::vector<bool> sync_choices(const ivb_problem* p) {
     return {false, true};
 }
 
+ivb_status default_tuning(ivb_problem* p);
+
 // Pick block size, blocks per SM, frame placement, threads per subdomain and
 // subdomains per grab (tile) by timing the bound kernel on the first
-// subdomains of the staged batch (results do not depend on the choice). The
-// timed index range is capped at two waves of the widest candidate grid, and a
-// candidate whose warm-up is already far slower than the best is not timed
-// again, so that tuning stays a small fraction of a few calls. Stage 1 times every
+// subdomains of the staged batch (results do not depend on the choice; a candidate
+// whose frames do not fit is left out). The timed index range is capped at two
+// waves of the widest candidate grid, and a candidate whose warm-up is already far
+// slower than the best is not timed again, so that tuning stays a small fraction of a few calls. Stage 1 times every
 // (threads per subdomain, block, blocks per SM, frame placement); stage 2
 // times larger grabs (4 and 16 passes per grab) for the best of stage 1.
 ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
@@ -336,6 +367,7 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
         p->tuned_interp = c.interp;
         ivb_status r = IVB_OK;
         if (reduce_units(p) > 0) r = ensure_frame(p, grid, c.block, reduce_units(p));
+        if (r == IVB_ENOMEM) { p->err.clear(); last_ms = 1e30f; return IVB_OK; }   // not a choice: left out
         if (r) return r;
         const int tile = c.tile_mult * pass_size(p, c.block, c.tpsub);
         // warm-up run, timed too: a candidate whose warm-up already takes 1.5x the
@@ -370,7 +402,7 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
         const TuneCand& c = cands[i];
         const bool same = i > 0 && cands[i - 1].interp == c.interp && cands[i - 1].sync == c.sync && cands[i - 1].tpsub == c.tpsub;
         if (!same) hopeless = false;
-        else if (cands[i - 1].block != c.block) hopeless = hopeless || size_ms > 2.f * best;
+        else if (cands[i - 1].block != c.block) hopeless = hopeless || (size_ms < 1e29f && size_ms > 2.f * best);
         if (!same || cands[i - 1].block != c.block) size_ms = 1e30f;
         if (hopeless) continue;
         st = time_one(c);
@@ -378,7 +410,7 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
     }
     // larger grabs: not for segmented kernels, whose passes are long and dealt out
     // evenly (a grab of four passes that fits the sample leaves others unbalanced)
-    if (!st && p->opt.tile <= 0 && (bc.interp || p->jit.state_units == 0)) {
+    if (!st && timed > 0 && p->opt.tile <= 0 && (bc.interp || p->jit.state_units == 0)) {
         const TuneCand base = bc;
         for (int mult : {4, 16}) {
             TuneCand c = base;
@@ -395,7 +427,11 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
     hdr[1] = g_end;
     CK(cudaMemcpyAsync(p->d_queue, p->h_queue, 16, cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));
-    if (st) return st;
+    if (!st && timed == 0) {   // no candidate's frames fit: the default shape, on as many blocks as do
+        st = default_tuning(p);
+        p->tuned = true;
+    }
+    if (st || timed == 0) return st;
     p->block = bc.block;
     p->bps = bc.bps;
     p->frame_smem = bc.smem;
@@ -409,8 +445,12 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
     p->tuned = true;
     p->cfg_ready = true;
     drop_graphs(p);
+    // the widest candidate's frames go back where the choice needs less
+    if ((size_t)p->sm_count * p->block * p->bps * reduce_units(p) * sizeof(double) < p->frame_bytes) free_frame(p);
     return IVB_OK;
 }
+
+bool wide(const ivb_problem* p, int units) { return wide_frames_fit(units * sizeof(double), p->sm_count, p->device_bytes); }
 
 ivb_status default_tuning(ivb_problem* p) {
     // a segmented kernel runs best as one block per SM: its warps then stream
@@ -419,9 +459,10 @@ ivb_status default_tuning(ivb_problem* p) {
     const bool seg = reduce_jit(p) && p->jit.state_units > 0;
     // the interpreter: frames in shared memory if four small blocks' fit, else 32
     // warps per SM (configuration 3, 941192 subdomains: 12.8 ms against 17.2 with 16)
-    const bool small = reduce_jit(p) || p->opt.frame_in_shared != -1 ||
+    const bool small = reduce_jit(p) || p->opt.frame_in_shared != -1 || !wide(p, frame_units(p)) ||
                        (smem_bytes(p, 128, 1) + 1024 <= (size_t)p->smem_optin && smem_bytes(p, 128, 1) * 4 <= 220 * 1024);
-    p->block = p->opt.block_threads > 0 ? p->opt.block_threads : seg ? p->jit.block_max : small ? 128 : 256;
+    const int seg_block = wide(p, p->jit.state_units) ? p->jit.block_max : std::min(512, p->jit.block_max);
+    p->block = p->opt.block_threads > 0 ? p->opt.block_threads : seg ? seg_block : small ? 128 : 256;
     p->bps = p->opt.blocks_per_sm > 0 ? p->opt.blocks_per_sm : seg && p->opt.block_threads <= 0 ? 1 : 4;
     const size_t bytes = smem_bytes(p, p->block, 1);
     if (reduce_jit(p)) p->frame_smem = 0;   // frames serve only the interpreter's store mode
@@ -667,6 +708,8 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     p->device = dev;
     CKC(cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev));
     CKC(cudaDeviceGetAttribute(&p->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    size_t unused = 0;
+    CKC(cudaMemGetInfo(&unused, &p->device_bytes));
     for (int m = 0; m < 4; ++m) CKC(set_bound_smem_limit(m, p->smem_optin - 1024));
     CKC(init_math_tables());
 
@@ -831,8 +874,8 @@ ivb_status bound_nodes_impl(ivb_problem* p, int32_t n_nodes, const double* boxes
             CK(cudaMemcpyAsync(p->d_queue, one.data(), one.size(), cudaMemcpyHostToDevice, s));
             const long long S = o2[1];
             const long long tiles = (S + p->block - 1) / p->block;
-            const int grid = (int)std::min<long long>(tiles, (long long)p->sm_count * p->bps);
-            if (reduce_units(p) > 0) st = ensure_frame(p, grid, p->block, reduce_units(p));
+            int grid = (int)std::min<long long>(tiles, (long long)p->sm_count * p->bps);
+            st = fit_frame(p, &grid, p->block, reduce_units(p));
             if (st) return st;
             CK(launch_init_keys(p->d_keys, p->d_queue, 1, p->n_out, p->d_counter, s));
             KParams K = make_params(p, p->frame_smem);
@@ -862,8 +905,8 @@ ivb_status bound_nodes_impl(ivb_problem* p, int32_t n_nodes, const double* boxes
             else if (!p->cfg_ready) st = default_tuning(p);
             if (st) return st;
         }
-        const int grid = p->sm_count * p->bps;
-        if (reduce_units(p) > 0) st = ensure_frame(p, grid, p->block, reduce_units(p));
+        int grid = p->sm_count * p->bps;
+        st = fit_frame(p, &grid, p->block, reduce_units(p));
         if (st) return st;
         const int tpsub = call_tpsub(p, total, (long long)grid * p->block);
         const int tile = tpsub == p->tpsub ? p->tile : pass_size(p, p->block, tpsub);
@@ -933,11 +976,12 @@ extern "C" ivb_status ivb_enclose(ivb_problem* p, const double* box, const int32
     // the store modes run the interpreter: in the shape of the reduce launches where these run it too,
     // else in the options' or its own
     const bool own = !reduce_jit(p);
-    const int block = own ? p->block : p->opt.block_threads > 0 ? p->opt.block_threads : 256;
+    const int block = own ? p->block : p->opt.block_threads > 0 ? p->opt.block_threads : wide(p, frame_units(p)) ? 256 : 128;
     const int bps = own ? p->bps : p->opt.blocks_per_sm > 0 ? p->opt.blocks_per_sm : 4;
     const int fs = own ? p->frame_smem : 0;
-    const int resident = p->sm_count * bps, grid = range_blocks(count, resident);   // dealt out evenly
-    st = ensure_frame(p, grid, block, frame_units(p));
+    const int resident = p->sm_count * bps;
+    int grid = range_blocks(count, resident);   // dealt out evenly
+    st = fit_frame(p, &grid, block, frame_units(p));
     if (st) return st;
     KParams K = make_params(p, fs);
     K.frame_units = frame_units(p);

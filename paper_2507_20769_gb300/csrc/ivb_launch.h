@@ -1,6 +1,7 @@
 // ivb_launch.h -- rules on the shape of the bounding launches (plain C++, no
 // CUDA: the CPU tests compile this file as it is).
 #pragma once
+#include <cstddef>
 
 namespace ivb {
 
@@ -18,6 +19,20 @@ inline int block_tpsub(int block, int wanted) { return groups_fit(block, wanted)
 inline int range_blocks(long long count, int resident) {
     const long long warps = (count + 31) / 32;
     return warps < resident ? (int)warps : resident;
+}
+
+// The library's own shapes run 1024 threads per SM where the frames of all of them
+// (`bytes` per thread) take at most a sixteenth of the device's memory (twice that of the 512 threads
+// that longer tapes get: 18 GB of 284 at 152 SMs, tapes of some 7000 entries per output).
+inline bool wide_frames_fit(size_t bytes, int sms, size_t device_bytes) {
+    return bytes * 1024 * (size_t)sms <= device_bytes / 16;
+}
+
+// Blocks to launch when memory is short: `blocks`, halved until get(blocks) succeeds;
+// 0 when it fails for one block too. The tile loops take any number of blocks.
+template <class Get> int blocks_that_fit(int blocks, Get get) {
+    while (blocks > 0 && !get(blocks)) blocks /= 2;
+    return blocks;
 }
 
 }  // namespace ivb

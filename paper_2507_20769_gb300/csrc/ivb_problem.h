@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cstdint>
 #include <string>
 
 #include "../../include/ivb.h"
@@ -43,8 +44,10 @@ struct ivb_problem {
     // frames
     double* d_frame = nullptr;
     size_t frame_bytes = 0;
+    size_t frame_most = SIZE_MAX;   // what the device had left for frames when an allocation failed
     // tuning
     int sm_count = 0, smem_optin = 0;
+    size_t device_bytes = 0;
     bool tuned = false;       // final configuration chosen
     bool cfg_ready = false;   // some configuration chosen (defaults while waiting for a batch worth tuning on)
     int block = 128, bps = 4, tile = 512, frame_smem = 0;

@@ -76,3 +76,29 @@ def test_stored_range_holds_frames_of_the_blocks_that_work(specialize):
         a, b, c = (np.asarray(o[k]) for o in out)
         assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
         assert np.array_equal(a.view(np.uint8), np.ascontiguousarray(c[7:8]).view(np.uint8))
+
+
+@pytest.mark.parametrize("autotune", [0, 1])
+def test_short_memory_runs_on_fewer_blocks(autotune):
+    """frames that do not fit beside what the program holds: fewer blocks, the same bits"""
+    t = W.config_tape(5)
+    boxes = W.bisection_frontier(t.root_box, 64, seed=2026)[:1]
+    splits = np.array([W.full_scale_splits(b, t.root_box) for b in boxes], np.int32)
+    with ivb.Problem(t, specialize=0, autotune=0) as p:
+        before = used()
+        ref = p.bound_nodes_ex(boxes, splits, want_hull=True)
+        full = used() - before
+        F = p.enclose(boxes[0], splits[0], first=5, count=20_000)[0]
+    assert full > 1 << 30
+    with ivb.Problem(t, specialize=0, autotune=autotune) as p:
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        hog = torch.empty(free - full * 6 // 10, dtype=torch.uint8, device="cuda:0")
+        try:
+            for _ in range(2):
+                assert_same(p.bound_nodes_ex(boxes, splits, want_hull=True), ref, "bounds")
+            G = p.enclose(boxes[0], splits[0], first=5, count=20_000)[0]
+        finally:
+            del hog
+            torch.cuda.empty_cache()
+    assert np.array_equal(F.view(np.uint8), G.view(np.uint8))

@@ -45,3 +45,24 @@ def test_blocks_of_a_range_all_get_work(rows):
     got = rows("for (long long c : {%s}) std::printf(\"%%lld %%d\\n\", c, range_blocks(c, 608));"
                % ", ".join(f"{c}LL" for c in counts))
     assert got == [[c, min(608, -(-c // 32))] for c in counts]
+
+
+def test_frames_when_memory_is_short(rows):
+    """a failing allocation halves the blocks until one succeeds, and gives up after one block"""
+    got = rows("for (int most : {0, 1, 2, 37, 303, 304, 607, 608, 5000}) { int calls = 0; "
+               "const int b = blocks_that_fit(608, [&](int g) { ++calls; return g <= most; }); "
+               'std::printf("%d %d %d\\n", most, b, calls); }')
+    for most, blocks, calls in got:
+        want = [b for b in (608, 304, 152, 76, 38, 19, 9, 4, 2, 1) if b <= most]
+        assert blocks == (want[0] if want else 0)
+        assert calls == 11 - max(1, len(want)), (most, calls)
+
+
+def test_default_shapes_keep_their_frames_small(rows):
+    """1024 threads per SM up to a sixteenth of the device's memory"""
+    mib = 284_208
+    got = rows("for (long long u : {1LL, 1680LL, 14000LL, 15000LL, 15500LL, 262000LL}) "
+               'std::printf("%%lld %%d\\n", u, (int)wide_frames_fit((size_t)u * 8, 152, (size_t)%dLL << 20));' % mib)
+    for units, wide in got:
+        assert wide == (units * 8 * 1024 * 152 <= (mib << 20) // 16), units
+    assert {w for _, w in got} == {0, 1}
