@@ -561,10 +561,6 @@ SegPolicy seg_policy(const ivb_options& o) {
     return pol;
 }
 
-// threads of the largest block of a segmented kernel: all that a register
-// budget allows on an SM, in whole groups of four warps
-int seg_block_max(int max_regs) { return std::min(1024, 65536 / max_regs / 128 * 128); }
-
 cudaError_t specialize_seg(ivb_problem* p, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
                            const std::vector<double>& consts, std::string* msg) {
     const int emu = p->opt.emulate >= 0 ? p->opt.emulate : kJitDefaultEmulate;

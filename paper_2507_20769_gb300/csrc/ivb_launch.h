@@ -14,6 +14,13 @@ inline bool groups_fit(int block, int groups) { return groups >= 1 && block % (3
 // where the block cannot be dealt out to that many groups
 inline int block_tpsub(int block, int wanted) { return groups_fit(block, wanted) ? wanted : 1; }
 
+// Threads of the largest block of a segmented kernel: all that a register budget
+// allows on an SM (registers come in eights), in whole groups of four warps.
+inline int seg_block_max(int max_regs) {
+    const int threads = 65536 / ((max_regs + 7) / 8 * 8) / 128 * 128;
+    return threads < 1024 ? threads : 1024;
+}
+
 // Blocks of a launch over `count` subdomains, of `resident` at most: a block takes a
 // warp of subdomains at least (even_tile), further blocks would only hold frames.
 inline int range_blocks(long long count, int resident) {

@@ -102,3 +102,16 @@ def test_short_memory_runs_on_fewer_blocks(autotune):
             del hog
             torch.cuda.empty_cache()
     assert np.array_equal(F.view(np.uint8), G.view(np.uint8))
+
+
+@pytest.mark.parametrize("seg_regs", [64, 73, 82, 100, 128, 170, 255])
+def test_every_register_budget_launches(reference, seg_regs):
+    """the default block of a segmented kernel fits an SM whatever the budget"""
+    with ivb.Problem(W.config_tape(2), specialize=3, autotune=0, seg_regs=seg_regs) as p:
+        c2 = p.bound_nodes_ex(W.config_tape(2).root_box[None], np.full((1, 4), 5, np.int32), want_hull=True)
+        assert p.get_tuning()["block_threads"] * -(-seg_regs // 8) * 8 <= 65536
+    with ivb.Problem(W.config_tape(2), specialize=0, autotune=0) as p:
+        assert_same(c2, p.bound_nodes_ex(W.config_tape(2).root_box[None], np.full((1, 4), 5, np.int32), want_hull=True),
+                    seg_regs)
+    with ivb.Problem(tape(), specialize=3, autotune=0, seg_regs=seg_regs) as p:
+        assert_same(bounds(p), reference, seg_regs)

@@ -66,3 +66,12 @@ def test_default_shapes_keep_their_frames_small(rows):
     for units, wide in got:
         assert wide == (units * 8 * 1024 * 152 <= (mib << 20) // 16), units
     assert {w for _, w in got} == {0, 1}
+
+
+def test_block_of_a_register_budget_fits_an_sm(rows):
+    got = rows('for (int r = 64; r <= 255; ++r) std::printf("%d %d\\n", r, seg_block_max(r));')
+    assert len(got) == 192
+    for regs, block in got:
+        per = -(-regs // 8) * 8
+        assert block % 128 == 0 and 256 <= block <= 1024 and block * per <= 65536, (regs, block)
+        assert block == 1024 or (block + 128) * per > 65536, (regs, block)
