@@ -154,7 +154,10 @@ typedef struct {
     int32_t seg_chunk;         /* segmented kernel: estimated FP64 issue
                                   slots per chunk (0 = default 320)         */
     int32_t seg_regs;          /* segmented kernel: register budget of every
-                                  chunk function, 64..255 (0 = default 64)  */
+                                  chunk function, 64..255; 0 (default): 64,
+                                  up to 128 where block_threads and
+                                  blocks_per_sm leave fewer than 1024
+                                  threads on an SM                          */
     int32_t threads_per_subdomain; /* segmented kernel with an own program
                                   per output: 1, 2 or 4 threads (in different
                                   warps of a block) share one subdomain, each

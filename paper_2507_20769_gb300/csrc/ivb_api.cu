@@ -555,7 +555,7 @@ SegPolicy seg_policy(const ivb_options& o) {
     if (o.seg_chunk > 0) pol.chunk_cost = o.seg_chunk;
     if (o.seg_ilp > 0) pol.ilp = o.seg_ilp;
     if (o.seg_outline >= 0) pol.outline = o.seg_outline;
-    if (o.seg_regs > 0) pol.max_regs = o.seg_regs;
+    pol.max_regs = seg_registers(o.seg_regs, o.block_threads, o.blocks_per_sm);
     const unsigned hc = std::thread::hardware_concurrency();
     pol.units = std::max(1, std::min(64, hc ? (int)hc : 8));
     return pol;

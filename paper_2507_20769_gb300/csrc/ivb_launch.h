@@ -14,6 +14,20 @@ inline bool groups_fit(int block, int groups) { return groups >= 1 && block % (3
 // where the block cannot be dealt out to that many groups
 inline int block_tpsub(int block, int wanted) { return groups_fit(block, wanted) ? wanted : 1; }
 
+// Register budget of a segmented kernel's functions. 64 lets 1024 threads fill an SM. Where
+// options fix a block that leaves fewer threads on an SM, their share of the registers, 128 at
+// most: more threads at 64 are slower in blocks that stream through the code separately, and the
+// same threads spill less with more (2 x 256 at 128 against 4 x 256 at 64: configuration 5, 2^19
+// subdomains, 75 and 113 ms; configuration 2, 16 x 16^4, 2.64 and 3.39 ms). Without
+// blocks_per_sm such a block counts as 512 threads per SM.
+inline int seg_registers(int seg_regs, int block_threads, int blocks_per_sm) {
+    if (seg_regs > 0) return seg_regs;
+    if (block_threads <= 0) return 64;
+    const int blocks = blocks_per_sm > 0 ? blocks_per_sm : block_threads < 512 ? 512 / block_threads : 1;
+    const long long regs = 65536 / ((long long)block_threads * blocks) / 8 * 8;
+    return regs < 64 ? 64 : regs > 128 ? 128 : (int)regs;
+}
+
 // Threads of the largest block of a segmented kernel: all that a register budget
 // allows on an SM (registers come in eights), in whole groups of four warps.
 inline int seg_block_max(int max_regs) {

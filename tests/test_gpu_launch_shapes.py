@@ -115,3 +115,18 @@ def test_every_register_budget_launches(reference, seg_regs):
                     seg_regs)
     with ivb.Problem(tape(), specialize=3, autotune=0, seg_regs=seg_regs) as p:
         assert_same(bounds(p), reference, seg_regs)
+
+
+@pytest.mark.parametrize("specialize", [3, -1])
+@pytest.mark.parametrize("block,per_sm,runs,regs", [(256, 0, 2, 128), (128, 0, 4, 128), (256, 2, 2, 128), (256, 4, 4, 64),
+                                                    (0, 2, 1, 64)])
+def test_fixed_shape_sets_the_register_budget(reference, specialize, block, per_sm, runs, regs):
+    """configuration 2's chunks use most of their budget: the former shapes keep 128 registers"""
+    t = W.config_tape(2)
+    with ivb.Problem(t, specialize=specialize, autotune=0, block_threads=block, blocks_per_sm=per_sm) as p:
+        r = p.bound_nodes_ex(t.root_box[None], np.full((1, 4), 5, np.int32), want_hull=True)
+        tun, spec = p.get_tuning(), p.get_specialization()
+    assert (tun["kernel"], tun["block_threads"], tun["blocks_per_sm"]) == (2, block or 1024, runs)
+    assert regs - 16 < spec["registers"] <= regs
+    with ivb.Problem(t, specialize=0, autotune=0) as p:
+        assert_same(r, p.bound_nodes_ex(t.root_box[None], np.full((1, 4), 5, np.int32), want_hull=True), block)

@@ -75,3 +75,23 @@ def test_block_of_a_register_budget_fits_an_sm(rows):
         per = -(-regs // 8) * 8
         assert block % 128 == 0 and 256 <= block <= 1024 and block * per <= 65536, (regs, block)
         assert block == 1024 or (block + 128) * per > 65536, (regs, block)
+
+
+def test_register_budget_follows_a_fixed_shape(rows):
+    """64 for the library's shapes; fixed ones get their threads' share of an SM, 64 to 128"""
+    got = {tuple(r[:3]): r[3] for r in rows(
+        'for (int s : {0, 100}) for (int b = 0; b <= 1024; b += 32) for (int k = 0; k <= 8; ++k) '
+        'std::printf("%d %d %d %d\\n", s, b, k, seg_registers(s, b, k));')}
+    for (seg_regs, block, per_sm), regs in got.items():
+        if seg_regs:
+            assert regs == seg_regs
+        elif block == 0:
+            assert regs == 64
+        else:
+            threads = block * (per_sm or max(1, 512 // block))
+            assert regs % 8 == 0 and 64 <= regs <= 128
+            assert regs == 64 or regs * threads <= 65536
+            assert regs == 128 or (regs + 8) * threads > 65536
+    # blocks up to 256 as before: two of 256, four of 128 at 128 registers
+    assert all(got[0, b, 0] == 128 for b in range(32, 257, 32))
+    assert got[0, 256, 2] == 128 and got[0, 256, 4] == 64 and got[0, 1024, 0] == 64 and got[0, 1024, 1] == 64
