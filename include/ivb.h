@@ -99,7 +99,13 @@ typedef struct {
                                   CUDA graph                                  */
     int32_t autotune;          /* 1 (default): pick block size, blocks per SM
                                   and tile on first use                       */
-    int32_t block_threads;     /* threads per block; 0 = tuned / default     */
+    int32_t block_threads;     /* threads per block, a multiple of 32; 0 =
+                                  tuned / default. Up to 512 with the
+                                  interpreter, 256 with specialize = 1 or 2,
+                                  1024 with the segmented kernel (as many as
+                                  seg_regs leaves registers for); with
+                                  specialize = -1 more than 256 where that
+                                  means 1 runs the interpreter              */
     int32_t blocks_per_sm;     /* resident blocks per SM; 0 = tuned/default  */
     int32_t tile;              /* subdomains a block grabs at a time; 0: as
                                   many as it has threads (smallest tail)   */

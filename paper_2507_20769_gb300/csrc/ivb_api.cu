@@ -333,7 +333,7 @@ ivb_status autotune(ivb_problem* p, long long total, cudaStream_t s) {
             for (int k : bpss) {
                 const int warps = b * k / 32;
                 if (warps < 4 || warps > 32 || !groups_fit(b, t)) continue;
-                if (b > (reduce_jit(p) ? (p->jit.state_units > 0 ? p->jit.block_max : 256) : 512)) continue;
+                if (b > (reduce_jit(p) ? p->jit.block_max : kInterpBlockMax)) continue;
                 for (int sm = 0; sm < 2; ++sm) {
                     const size_t bytes = smem_bytes(p, b, sm);
                     if (sm && (reduce_jit(p) || bytes + 1024 > (size_t)p->smem_optin || bytes * k > 220 * 1024)) continue;
@@ -463,6 +463,7 @@ ivb_status default_tuning(ivb_problem* p) {
                        (smem_bytes(p, 128, 1) + 1024 <= (size_t)p->smem_optin && smem_bytes(p, 128, 1) * 4 <= 220 * 1024);
     const int seg_block = wide(p, p->jit.state_units) ? p->jit.block_max : std::min(512, p->jit.block_max);
     p->block = p->opt.block_threads > 0 ? p->opt.block_threads : seg ? seg_block : small ? 128 : 256;
+    if (!reduce_jit(p)) p->block = std::min(p->block, kInterpBlockMax);   // asked of a kernel that did not compile
     p->bps = p->opt.blocks_per_sm > 0 ? p->opt.blocks_per_sm : seg && p->opt.block_threads <= 0 ? 1 : 4;
     const size_t bytes = smem_bytes(p, p->block, 1);
     if (reduce_jit(p)) p->frame_smem = 0;   // frames serve only the interpreter's store mode
@@ -555,7 +556,7 @@ SegPolicy seg_policy(const ivb_options& o) {
     if (o.seg_chunk > 0) pol.chunk_cost = o.seg_chunk;
     if (o.seg_ilp > 0) pol.ilp = o.seg_ilp;
     if (o.seg_outline >= 0) pol.outline = o.seg_outline;
-    pol.max_regs = seg_registers(o.seg_regs, o.block_threads, o.blocks_per_sm);
+    pol.max_regs = seg_budget(o.seg_regs, o.block_threads, o.blocks_per_sm);
     const unsigned hc = std::thread::hardware_concurrency();
     pol.units = std::max(1, std::min(64, hc ? (int)hc : 8));
     return pol;
@@ -656,8 +657,8 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
         return fail(nullptr, IVB_EINVAL, "grad_mode must be IVB_GRAD_FORWARD or IVB_GRAD_ADJOINT");
     if (o.form < 0 || o.form > 2) return fail(nullptr, IVB_EINVAL, "form must be 0, 1 or 2");
     if (o.max_nodes < 1 || o.max_nodes > (1 << 20)) return fail(nullptr, IVB_EINVAL, "max_nodes must be in [1, 2^20]");
-    if (o.block_threads < 0 || o.block_threads > 512 || (o.block_threads % 32))
-        return fail(nullptr, IVB_EINVAL, "block_threads must be a multiple of 32 up to 512 (0 = auto)");
+    if (o.block_threads < 0 || (o.block_threads % 32))
+        return fail(nullptr, IVB_EINVAL, "block_threads must be a multiple of 32 (0 = auto)");
     if (o.specialize < -1 || o.specialize > 3) return fail(nullptr, IVB_EINVAL, "specialize must be -1, 0, 1, 2 or 3");
     if (o.specialize == 3 && o.grad_mode != IVB_GRAD_ADJOINT)
         return fail(nullptr, IVB_EINVAL, "specialize = 3 (segmented) needs grad_mode IVB_GRAD_ADJOINT");
@@ -672,8 +673,6 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     if (o.seg_regs != 0 && (o.seg_regs < 64 || o.seg_regs > 255))
         return fail(nullptr, IVB_EINVAL, "seg_regs must be 0 or in [64, 255]");
     if (o.emulate < -1 || o.emulate > 15) return fail(nullptr, IVB_EINVAL, "emulate must be -1 or a bitmask in [0, 15]");
-    if (o.specialize && o.block_threads > kJitBlockMax)
-        return fail(nullptr, IVB_EINVAL, "block_threads above 256 with a tape-specialised kernel");
     ivb_problem* p = new ivb_problem();
     p->opt = o;
     std::vector<Ins> ins;
@@ -681,6 +680,19 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     std::vector<double> consts;
     e = compile_tape(tape, p->P, ins, rins, consts);
     if (!e.empty()) { delete p; return fail(nullptr, IVB_ENOTSUP, e); }
+    // the kernel, and the largest block that options can ask of it: every shape that the
+    // autotuner reports can be asked for
+    long long ops = 0;
+    for (int k = 0; k < IVB_CNT_N; ++k) ops += o.grad_mode == IVB_GRAD_ADJOINT ? p->P.cnt_adj[k] : p->P.cnt_fwd[k];
+    const bool small = ops / 2 <= (o.grad_mode == IVB_GRAD_ADJOINT ? kSegMinOps : kJitAutoMaxOps);
+    const bool seg = o.specialize == 3 || (o.specialize == -1 && !small && o.grad_mode == IVB_GRAD_ADJOINT);
+    const int most = seg ? seg_block_limit(o.seg_regs) : o.specialize >= 1 ? kCompiledBlockMax : kInterpBlockMax;
+    if (o.block_threads > most) {
+        delete p;
+        return fail(nullptr, IVB_EINVAL, "block_threads above " + std::to_string(most) + " with this kernel");
+    }
+    // by the library's choice, a block beyond the compiled kernel's runs the interpreter
+    const bool compiled = seg || o.specialize >= 1 || (o.specialize == -1 && small && o.block_threads <= kCompiledBlockMax);
     p->n = tape->n_vars;
     p->n_out = tape->n_outputs;
     p->obj = p->P.obj;
@@ -769,28 +781,21 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     CKC(cudaMalloc(&p->d_counter, sizeof(unsigned long long)));
     CKC(cudaMalloc(&p->d_out, OutLayout(p->max_nodes, p->n_out).bytes));
     CKC(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
-    if (o.specialize) {
-        const int64_t* cnt = o.grad_mode == IVB_GRAD_ADJOINT ? p->P.cnt_adj : p->P.cnt_fwd;
-        long long ops = 0;
-        for (int k = 0; k < IVB_CNT_N; ++k) ops += cnt[k];
-        const bool small = ops / 2 <= (o.grad_mode == IVB_GRAD_ADJOINT ? kSegMinOps : kJitAutoMaxOps);
-        const bool seg = o.specialize == 3 || (o.specialize == -1 && !small && o.grad_mode == IVB_GRAD_ADJOINT);
-        if (o.specialize >= 1 || small || seg) {
-            const int mode = o.grad_mode == IVB_GRAD_ADJOINT ? KM_ADJ_REDUCE : KM_FWD_REDUCE;
-            std::string msg;
-            const cudaError_t ce = seg ? specialize_seg(p, ins, rins, consts, &msg)
-                                       : specialize(p, ins, rins, consts, mode, &msg);
-            if (ce != cudaSuccess || !msg.empty()) {
-                jit_unload(p->jit);
-                if (o.specialize >= 1) {
-                    ivb_destroy(p);
-                    if (ce != cudaSuccess)
-                        return fail(nullptr, ce == cudaErrorMemoryAllocation ? IVB_ENOMEM : IVB_ECUDA,
-                                    std::string("loading the tape-specialised kernel: ") + cudaGetErrorString(ce));
-                    return fail(nullptr, IVB_ENOTSUP, msg);
-                }
-                cudaGetLastError();
+    if (compiled) {
+        const int mode = o.grad_mode == IVB_GRAD_ADJOINT ? KM_ADJ_REDUCE : KM_FWD_REDUCE;
+        std::string msg;
+        const cudaError_t ce = seg ? specialize_seg(p, ins, rins, consts, &msg)
+                                   : specialize(p, ins, rins, consts, mode, &msg);
+        if (ce != cudaSuccess || !msg.empty()) {
+            jit_unload(p->jit);
+            if (o.specialize >= 1) {
+                ivb_destroy(p);
+                if (ce != cudaSuccess)
+                    return fail(nullptr, ce == cudaErrorMemoryAllocation ? IVB_ENOMEM : IVB_ECUDA,
+                                std::string("loading the tape-specialised kernel: ") + cudaGetErrorString(ce));
+                return fail(nullptr, IVB_ENOTSUP, msg);
             }
+            cudaGetLastError();
         }
     }
 #undef CKC
@@ -972,7 +977,8 @@ extern "C" ivb_status ivb_enclose(ivb_problem* p, const double* box, const int32
     // the store modes run the interpreter: in the shape of the reduce launches where these run it too,
     // else in the options' or its own
     const bool own = !reduce_jit(p);
-    const int block = own ? p->block : p->opt.block_threads > 0 ? p->opt.block_threads : wide(p, frame_units(p)) ? 256 : 128;
+    const int asked = std::min(p->opt.block_threads, kInterpBlockMax);
+    const int block = own ? p->block : asked > 0 ? asked : wide(p, frame_units(p)) ? 256 : 128;
     const int bps = own ? p->bps : p->opt.blocks_per_sm > 0 ? p->opt.blocks_per_sm : 4;
     const int fs = own ? p->frame_smem : 0;
     const int resident = p->sm_count * bps;

@@ -15,6 +15,7 @@
 
 #include "ivb_internal.h"
 #include "ivb_kparams.h"
+#include "ivb_launch.h"
 
 namespace ivb {
 
@@ -27,7 +28,7 @@ namespace ivb {
 // (configuration 2, 16 nodes x 16^4: 2.06 ms against 2.75) and compiles in a
 // tenth of the time; at 231 operations and two outputs a small call takes 52 us
 // against 65 (call_tpsub); below, there is little to cut.
-constexpr int kJitBlockMax = 256, kJitMinBlocks = 2, kJitAutoMaxOps = 1024, kSegMinOps = 128;
+constexpr int kJitBlockMax = kCompiledBlockMax, kJitMinBlocks = 2, kJitAutoMaxOps = 1024, kSegMinOps = 128;
 // chunks from which a segmented kernel keeps its warps on one chunk (below, the
 // autotuner times both). Warps that drift apart stream through the code
 // separately, and a sample of uniform subdomains does not show it: 306 chunks 56

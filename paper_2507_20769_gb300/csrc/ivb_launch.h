@@ -5,6 +5,9 @@
 
 namespace ivb {
 
+// threads of the largest block of each bounding kernel
+constexpr int kInterpBlockMax = 512, kCompiledBlockMax = 256, kSegBlockMax = 1024;
+
 // A block's threads can form `groups` groups that share each subdomain's outputs:
 // every group is whole warps, so that no warp runs two groups' programs (its
 // reductions and, with chunk synchronisation, its named barriers want whole warps).
@@ -29,10 +32,19 @@ inline int seg_registers(int seg_regs, int block_threads, int blocks_per_sm) {
 }
 
 // Threads of the largest block of a segmented kernel: all that a register budget
-// allows on an SM (registers come in eights), in whole groups of four warps.
+// allows on an SM, in whole groups of four warps (one to each of its four register files; registers
+// come in eights).
 inline int seg_block_max(int max_regs) {
     const int threads = 65536 / ((max_regs + 7) / 8 * 8) / 128 * 128;
-    return threads < 1024 ? threads : 1024;
+    return threads < kSegBlockMax ? threads : kSegBlockMax;
+}
+// the largest block that options can ask of it
+inline int seg_block_limit(int seg_regs) { return seg_regs > 0 ? seg_block_max(seg_regs) : kSegBlockMax; }
+// the budget of a kernel built for blocks of `block_threads` (0: the library's)
+inline int seg_budget(int seg_regs, int block_threads, int blocks_per_sm) {
+    const int regs = seg_registers(seg_regs, block_threads, blocks_per_sm);
+    if (block_threads <= seg_block_max(regs)) return regs;
+    return 65536 / ((block_threads + 127) / 128 * 128) / 8 * 8;
 }
 
 // Blocks of a launch over `count` subdomains, of `resident` at most: a block takes a

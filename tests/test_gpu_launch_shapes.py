@@ -130,3 +130,36 @@ def test_fixed_shape_sets_the_register_budget(reference, specialize, block, per_
     assert regs - 16 < spec["registers"] <= regs
     with ivb.Problem(t, specialize=0, autotune=0) as p:
         assert_same(r, p.bound_nodes_ex(t.root_box[None], np.full((1, 4), 5, np.int32), want_hull=True), block)
+
+
+@pytest.mark.parametrize("opts,which", [(dict(specialize=-1), 2), (dict(specialize=3), 2), (dict(specialize=1), 2),
+                                        (dict(specialize=0), 2), (dict(specialize=-1), "small"),
+                                        (dict(specialize=-1, grad_mode="forward"), 2)])
+def test_the_tuned_shape_can_be_asked_for(opts, which):
+    """what get_tuning reports goes back in as options: the same launch, the same bits"""
+    t = W.config_tape(2) if which == 2 else W.random_problem(4, 14, 0, W.OPS_ALL, [[-2, 2]] * 4, 8, "small")
+    boxes = W.bisection_frontier(t.root_box, 8, seed=20)
+    splits = np.full((8, t.n_vars), 14, np.int32)
+    with ivb.Problem(t, **opts) as p:
+        ref = p.bound_nodes_ex(boxes, splits, want_hull=True)
+        tun = p.get_tuning()
+        assert tun["candidates"] > 0
+    fixed = {k: tun[k] for k in ("block_threads", "blocks_per_sm", "tile", "frame_in_shared", "threads_per_subdomain")}
+    with ivb.Problem(t, seg_sync=tun["chunk_sync"], **dict(opts, **fixed)) as p:
+        r = p.bound_nodes_ex(boxes, splits, want_hull=True)
+        again = p.get_tuning()
+        if tun["kernel"] == 0 and p.get_specialization()["active"]:
+            fixed.pop("frame_in_shared")   # the compiled kernel has none
+    assert {k: again[k] for k in fixed} == {k: tun[k] for k in fixed}
+    assert_same(r, ref, fixed)
+
+
+@pytest.mark.parametrize("block", [288, 512, 672, 992, 1024])
+def test_segmented_kernel_at_any_block(reference, block):
+    with ivb.Problem(tape(), specialize=3, seg_chunk=24, block_threads=block) as p:
+        assert_same(bounds(p), reference, block)
+        assert p.get_tuning()["block_threads"] == block
+        box, splits = np.array([[-2.0, 2.0]] * 2), np.array([70, 60], np.int32)
+        F = p.enclose(box, splits, first=33, count=4001)[0]
+    with ivb.Problem(tape(), specialize=0, autotune=0) as p:
+        assert np.array_equal(F.view(np.uint8), p.enclose(box, splits, first=33, count=4001)[0].view(np.uint8))

@@ -95,3 +95,36 @@ def test_register_budget_follows_a_fixed_shape(rows):
     # blocks up to 256 as before: two of 256, four of 128 at 128 registers
     assert all(got[0, b, 0] == 128 for b in range(32, 257, 32))
     assert got[0, 256, 2] == 128 and got[0, 256, 4] == 64 and got[0, 1024, 0] == 64 and got[0, 1024, 1] == 64
+
+
+def test_segmented_kernel_is_built_for_the_block_asked_for(rows):
+    got = rows('for (int b = 0; b <= 1024; b += 32) for (int k = 0; k <= 8; ++k) { const int r = seg_budget(0, b, k); '
+               'std::printf("%d %d %d %d %d\\n", b, k, r, seg_block_max(r), seg_registers(0, b, k)); }')
+    for block, per_sm, regs, most, wanted in got:
+        assert block <= most and 64 <= regs <= wanted, (block, per_sm)
+        assert regs == wanted or -(-block // 128) * 128 * (regs + 8) > 65536, (block, per_sm)
+
+
+@pytest.mark.parametrize("opts,big_tape,most", [
+    (dict(specialize=0), True, 512), (dict(specialize=1), True, 256), (dict(specialize=2), False, 256),
+    (dict(specialize=3), True, 1024), (dict(specialize=3), False, 1024), (dict(specialize=-1), True, 1024),
+    (dict(specialize=-1), False, 512), (dict(specialize=-1, grad_mode="forward"), True, 512),
+    (dict(specialize=3, seg_regs=128), True, 512), (dict(specialize=3, seg_regs=100), True, 512),
+    (dict(specialize=3, seg_regs=255), True, 256)])
+def test_largest_block_that_options_can_ask_for(opts, big_tape, most):
+    """every shape that the autotuner can report is accepted, and nothing a kernel is not built for
+    (invalid options are refused before the device is touched: no GPU needed)"""
+    from paper_2507_20769_gb300 import build as B
+    from paper_2507_20769_gb300 import workloads as W
+    B.build()
+    from paper_2507_20769_gb300 import ivb
+    t = W.random_problem(2, 40 if big_tape else 6, 2 if big_tape else 0, W.OPS_RATIONAL, [[-2, 2]] * 2, 7, "blocks")
+
+    def refused(block):
+        try:
+            ivb.Problem(t, block_threads=block, **opts).destroy()
+        except ivb.IvbError as e:
+            return e.status == ivb.IVB_EINVAL
+        return False
+    assert not refused(most) and not refused(32)
+    assert refused(most + 32) and refused(most - 1) and refused(-32)
