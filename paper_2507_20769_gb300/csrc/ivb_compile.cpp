@@ -364,8 +364,7 @@ void interpreter_programs(const HostProgram& P, const std::vector<Ins>& ins, con
             const Ins& I = ins[i];
             const uint32_t op = I.w0 & 31u, ak = (I.w0 >> 5) & 3u, bk = (I.w0 >> 7) & 3u, ai = I.w1 & 0xFFFFu, bi = I.w1 >> 16;
             XIns& X = xins[to + i - begin];
-            X.w = op | (ak == K_CONST ? 1u << 5 : 0u) | (bk == K_CONST || bk == K_NONE ? 1u << 6 : 0u) |
-                  (ak == K_VAR ? 1u << 7 | (ai & 0xFFu) << 16 : 0u) | (bk == K_VAR ? 1u << 8 | (bi & 0xFFu) << 24 : 0u);
+            X.w = op | (ak == K_VAR ? 1u << 7 : 0u) | (bk == K_VAR ? 1u << 8 : 0u);
             X.dst = word(K_SLOT, I.w0 >> 16, base, rec, point);
             X.a = word(ak, ai, base, rec, point);
             X.b = bk == K_NONE ? X.a : word(bk, bi, base, rec, point);

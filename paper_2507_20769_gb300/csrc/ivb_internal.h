@@ -52,7 +52,7 @@ struct RIns {
 // instruction before.
 constexpr uint32_t kOpConst = 0x80000000u, kOpPoint = 0x40000000u, kOpLast = 0x20000000u, kOpIndex = 0x1FFFFFFFu;
 struct alignas(16) XIns {
-    // w = op[0:5) | a const[5] | b const or none[6] | a variable[7] | b variable[8] | a index[16:24) | b index[24:32)
+    // w = op[0:5) | a variable[7] | b variable[8]
     uint32_t w, dst, a, b;
 };
 constexpr uint32_t kAdjLast = 1u << 9;   // the result's adjoint is what the instruction before stored last
