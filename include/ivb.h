@@ -443,7 +443,10 @@ ivb_status ivb_specialize_compile(const ivb_tape* tape, int32_t grad_mode, int32
  * Interval products count two directed multiplies (sign-case selection); a
  * product added to an accumulator (adjoint accumulation, tangent rules, the
  * Mean Value Form sum) is one fused multiply-add per end, counted as a
- * multiply with no separate add. */
+ * multiply with no separate add. In forward mode the tangent rules count all
+ * n_vars directions; the interpreter leaves out those that an entry does not
+ * depend on. Doublings, quotients, reciprocals, roots, exp and log are counted
+ * although the kernels run them on the integer pipes. */
 enum {
     IVB_CNT_ADDSUB = 0, IVB_CNT_MUL = 1, IVB_CNT_DIV = 2, IVB_CNT_RCP = 3,
     IVB_CNT_SQRT = 4, IVB_CNT_EXP = 5, IVB_CNT_LOG = 6, IVB_CNT_RN = 7, IVB_CNT_N = 8

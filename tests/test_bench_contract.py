@@ -98,3 +98,43 @@ def test_roofline_fraction_is_algorithmic_endpoint_operations_over_the_fp64_peak
     assert abs(rf["peak"] - peak / 1e9) <= 1e-9
     rf2 = b.roofline_block(FakeProblem(), subs, step_s, {"sm_mhz": None}, 0)   # no clock sample: maximum clock
     assert abs(rf2["peak"] - peak / 1e9) <= 1e-9
+
+
+def test_pipe_busy_counts_only_what_the_kernel_leaves_on_the_fp64_pipe(monkeypatch):
+    """counted by hand for 2 x0 + x0 x1, sqr(x0) / x1 and a sum of two quotients' shared
+    operand; and the busy fraction is that count over the measured DFMA rate"""
+    import types
+    import torch
+    import problems as P
+    from paper_2507_20769_gb300 import ivb
+    b = _load_bench()
+    Bd = P.Builder(2)
+    x0, x1 = Bd.x(0), Bd.x(1)
+    Bd.output(Bd.add(Bd.mul(Bd.const(2.0), x0), Bd.mul(x0, x1)), P.KIND_OBJ)
+    t = Bd.tape([[-1.0, 1.0]] * 2, "by hand")
+    # decode 12, X - c 4, MVF 4; sum 4; x0 x1: 4 + 2 + 2; 2 x0: values none, its (second) contribution 2
+    assert b.fp64_pipe_ops(t, "segmented") == 20 + 4 + 8 + 2
+    # 2 x0 is a product like any other; two additions into G
+    assert b.fp64_pipe_ops(t, "interpreter") == 20 + 4 + 8 + 6 + 4
+    Bd = P.Builder(2)
+    x0, x1 = Bd.x(0), Bd.x(1)
+    Bd.output(Bd.div(Bd.sqr(x0), x1), P.KIND_OBJ)
+    t = Bd.tape([[1.0, 2.0]] * 2, "by hand")
+    # quotient on the integer pipes: W R, W V and its product with R; square 4 + 2
+    assert b.fp64_pipe_ops(t, "segmented") == 20 + 6 + 6
+
+    class FakeProblem:
+        def op_counts(self):
+            return {"mul": 100}
+
+        def get_segmentation(self):
+            return {"recomputed": 0}
+
+        def get_tuning(self):
+            return {"kernel": 2}
+
+    monkeypatch.setattr(torch.cuda, "get_device_properties", lambda dev: types.SimpleNamespace(multi_processor_count=152))
+    monkeypatch.setattr(b, "traffic_for", lambda subs, which: None)
+    monkeypatch.setattr(ivb, "ivb_fp64_probe", lambda name: 500e9)
+    rf = b.roofline_block(FakeProblem(), 1 << 20, 0.5, {"sm_mhz": 2070.0}, 0, probes=True, tape=t)
+    assert abs(rf["pipe_busy_frac"] - 32 * (1 << 20) / 0.5 / 500e9) <= 1e-12
