@@ -196,7 +196,9 @@ typedef struct {
                                   per statement); 2 only * sqr and the fused
                                   accumulation (+ and - inline); 0 inlines
                                   them all; -1 (default): the library's
-                                  choice, now 2                             */
+                                  choice, now 2 (1 where `emulate` covers
+                                  sums and the tape has more than 1024
+                                  interval operations per subdomain)        */
 } ivb_options;
 
 typedef struct ivb_problem ivb_problem;

@@ -548,14 +548,22 @@ struct Outputs {
 
 // ======================================================================= ABI
 
-// generate, compile and load the tape-specialised reduce kernel
+// interval operations per subdomain
+long long interval_ops(const HostProgram& P, int grad_mode) {
+    const int64_t* cnt = grad_mode == IVB_GRAD_ADJOINT ? P.cnt_adj : P.cnt_fwd;
+    long long ends = 0;
+    for (int k = 0; k < IVB_CNT_N; ++k) ends += cnt[k];
+    return ends / 2;
+}
+
 // segmentation options of a problem
-SegPolicy seg_policy(const ivb_options& o) {
+SegPolicy seg_policy(const ivb_options& o, const HostProgram& P) {
     SegPolicy pol;
     if (o.recompute >= 0) pol.recompute = o.recompute;
     if (o.seg_chunk > 0) pol.chunk_cost = o.seg_chunk;
     if (o.seg_ilp > 0) pol.ilp = o.seg_ilp;
-    if (o.seg_outline >= 0) pol.outline = o.seg_outline;
+    const int emu = o.emulate >= 0 ? o.emulate : kJitDefaultEmulate;
+    pol.outline = seg_outline_for(o.seg_outline, emu, interval_ops(P, IVB_GRAD_ADJOINT));
     pol.max_regs = seg_budget(o.seg_regs, o.block_threads, o.blocks_per_sm);
     const unsigned hc = std::thread::hardware_concurrency();
     pol.units = std::max(1, std::min(64, hc ? (int)hc : 8));
@@ -565,7 +573,7 @@ SegPolicy seg_policy(const ivb_options& o) {
 cudaError_t specialize_seg(ivb_problem* p, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
                            const std::vector<double>& consts, std::string* msg) {
     const int emu = p->opt.emulate >= 0 ? p->opt.emulate : kJitDefaultEmulate;
-    const SegPolicy pol = seg_policy(p->opt);
+    const SegPolicy pol = seg_policy(p->opt, p->P);
     const int block_max = seg_block_max(pol.max_regs);
     const SegSource src = jit_seg_source(p->P, ins, rins, consts, block_max, emu, p->opt.form, pol);
     std::vector<char> cubin;
@@ -600,6 +608,7 @@ cudaError_t specialize_seg(ivb_problem* p, const std::vector<Ins>& ins, const st
     return cudaSuccess;
 }
 
+// generate, compile and load the tape-specialised reduce kernel
 cudaError_t specialize(ivb_problem* p, const std::vector<Ins>& ins, const std::vector<RIns>& rins,
                        const std::vector<double>& consts, int mode, std::string* msg) {
     const int emu = p->opt.emulate >= 0 ? p->opt.emulate : kJitDefaultEmulate;
@@ -682,9 +691,7 @@ extern "C" ivb_status ivb_create_problem(const ivb_tape* tape, const ivb_options
     if (!e.empty()) { delete p; return fail(nullptr, IVB_ENOTSUP, e); }
     // the kernel, and the largest block that options can ask of it: every shape that the
     // autotuner reports can be asked for
-    long long ops = 0;
-    for (int k = 0; k < IVB_CNT_N; ++k) ops += o.grad_mode == IVB_GRAD_ADJOINT ? p->P.cnt_adj[k] : p->P.cnt_fwd[k];
-    const bool small = ops / 2 <= (o.grad_mode == IVB_GRAD_ADJOINT ? kSegMinOps : kJitAutoMaxOps);
+    const bool small = interval_ops(p->P, o.grad_mode) <= (o.grad_mode == IVB_GRAD_ADJOINT ? kSegMinOps : kJitAutoMaxOps);
     const bool seg = o.specialize == 3 || (o.specialize == -1 && !small && o.grad_mode == IVB_GRAD_ADJOINT);
     const int most = seg ? seg_block_limit(o.seg_regs) : o.specialize >= 1 ? kCompiledBlockMax : kInterpBlockMax;
     if (o.block_threads > most) {
@@ -1175,7 +1182,7 @@ extern "C" ivb_status ivb_specialize_compile(const ivb_tape* tape, int32_t grad_
         ivb_options o;
         ivb_options_default(&o);
         if (compact == 4) o.seg_ilp = 2;
-        const SegPolicy pol = seg_policy(o);
+        const SegPolicy pol = seg_policy(o, P);
         const SegSource src = jit_seg_source(P, ins, rins, consts, seg_block_max(pol.max_regs),
                                              compact == 4 ? 15 : kJitDefaultEmulate, 0, pol);
         e = jit_seg_compile(src, pol.max_regs, cubin, tables, seconds, &regs, &spill);

@@ -47,6 +47,15 @@ inline int seg_budget(int seg_regs, int block_threads, int blocks_per_sm) {
     return 65536 / ((block_threads + 127) / 128 * 128) / 8 * 8;
 }
 
+// Short operations of a segmented kernel out of line (options seg_outline and emulate, interval
+// operations per subdomain): by the library's choice the products. Sums emulated on the integer
+// pipes are long too, and inline in a large tape they quadruple its compile time and slow it down
+// (configuration 5, emulate = 12: 73 ms and 6 s with all out of line, 98 ms and 24 s with the
+// products alone; configuration 2, emulate = 15: 5.3 and 4.0 ms, 0.7 and 1.8 s).
+inline int seg_outline_for(int option, int emulate, long long ops) {
+    return option >= 0 ? option : (emulate & 12) && ops > 1024 ? 1 : 2;
+}
+
 // Blocks of a launch over `count` subdomains, of `resident` at most: a block takes a
 // warp of subdomains at least (even_tile), further blocks would only hold frames.
 inline int range_blocks(long long count, int resident) {

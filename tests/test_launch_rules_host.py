@@ -128,3 +128,11 @@ def test_largest_block_that_options_can_ask_for(opts, big_tape, most):
         return False
     assert not refused(most) and not refused(32)
     assert refused(most + 32) and refused(most - 1) and refused(-32)
+
+
+def test_emulated_sums_of_large_tapes_are_called_out_of_line(rows):
+    got = rows('for (int o = -1; o <= 2; ++o) for (int e = 0; e < 16; ++e) for (long long k : {1LL, 1024LL, 1025LL, 99999LL}) '
+               'std::printf("%d %d %lld %d\\n", o, e, k, seg_outline_for(o, e, k));')
+    assert len(got) == 256
+    for option, emulate, ops, out in got:
+        assert out == (option if option >= 0 else 1 if emulate >= 4 and ops > 1024 else 2)
