@@ -170,10 +170,14 @@ typedef struct {
                                   running the programs of a group of its
                                   outputs; 0 (default): chosen by the
                                   autotuner among those compiled, and more
-                                  of them in calls of few subdomains. Runs
-                                  with 1 where block_threads is not a
-                                  multiple of 32 times the number (each group
-                                  is whole warps)                           */
+                                  of them in calls of few subdomains, where
+                                  the interpreter shares the outputs among
+                                  warp groups too; any other value fixes the
+                                  number for calls of every size (the
+                                  interpreter then runs with 1). Runs with 1
+                                  where block_threads is not a multiple of 32
+                                  times the number (each group is whole
+                                  warps)                                    */
     int32_t seg_sync;          /* segmented kernel: 1 the warps of a thread
                                   group wait for each other after every chunk
                                   function (they then run the same code and
@@ -380,7 +384,11 @@ ivb_status ivb_host_gradient(const ivb_tape* tape, const double* box, int32_t ou
                              double* G);
 
 /* Tuning actually used by the batched path after autotuning (may be NULL):
- * block threads, blocks per SM, tile, frame in shared (0/1). */
+ * block threads, blocks per SM, tile, frame in shared (0/1). This and
+ * ivb_get_tuning_ex report the launch of calls that fill the device: smaller
+ * calls share each subdomain among more threads (threads_per_subdomain), and
+ * where memory is short a launch has fewer blocks. Each value can be given
+ * back as the option of its name (chunk_sync as seg_sync). */
 ivb_status ivb_get_tuning(ivb_problem* p, int32_t* block_threads, int32_t* blocks_per_sm,
                           int32_t* tile, int32_t* frame_in_shared);
 

@@ -24,10 +24,12 @@ namespace ivb {
 // kJitAutoMaxOps interval operations per subdomain as one program (beyond that,
 // compile time grows to tens of seconds and the interpreter was within 5 % on
 // the configurations measured). In adjoint mode the segmented kernel takes
-// over from kSegMinOps on: with 32 warps per SM it is ahead at 620 operations
-// (configuration 2, 16 nodes x 16^4: 2.06 ms against 2.75) and compiles in a
-// tenth of the time; at 231 operations and two outputs a small call takes 52 us
-// against 65 (call_tpsub); below, there is little to cut.
+// over from kSegMinOps on, where it is ahead in calls of every size and compiles in half to a
+// tenth of the time. Segmented against compact, 2^20 and 1024 subdomains: 620 operations (16 x 16^4)
+// 2.07 ms against 2.77; 209 and four outputs 0.74 ms and 62 us against 0.91 and 83; 171 and one output
+// 0.61 ms and 75 us against 0.68 and 78. Below the line large calls still gain 4 to 12 % (122
+// operations 0.47 ms against 0.54, 62 0.23 against 0.25) but small ones lose (122 69 us against 67, 39 56
+// against 52), so the compact kernel stays there.
 constexpr int kJitBlockMax = kCompiledBlockMax, kJitMinBlocks = 2, kJitAutoMaxOps = 1024, kSegMinOps = 128;
 // chunks from which a segmented kernel keeps its warps on one chunk (below, the
 // autotuner times both). Warps that drift apart stream through the code
@@ -36,10 +38,9 @@ constexpr int kJitBlockMax = kCompiledBlockMax, kJitMinBlocks = 2, kJitAutoMaxOp
 // (configuration 3), but 37 and 45 ms on 256 uneven nodes; 12 chunks 4.4 and 4.0 ms
 constexpr int kSegSyncChunks = 20;
 // endpoint operations emulated on the integer pipes by default (ivb_iv.cuh
-// policy bits): none -- on configuration 2 no policy beat the FP64 pipe alone
-// by more than the noise (the kernel runs at its 128-register cap with 16
-// warps per SM and long dependency chains, so the emulation's latency, not
-// the FP64 pipe, ends up on the critical path)
+// policy bits): none. The integer ALU is half busy with the selects and the fixed-point
+// primitives, so every policy is slower (2^19 subdomains of configuration 5: 48.9 ms with none, 54.6
+// with 1, 62 with 3, 73 with 12; configuration 2, 16 x 16^4: 2.05, 2.36 with 1, 4.0 with 15)
 constexpr int kJitDefaultEmulate = 0;
 
 struct JitKernel {
@@ -75,14 +76,16 @@ struct SegPolicy {
     int recompute = 0;           // measured fastest: recomputation adds FP64 work, the state area streams with room to spare
     int units = 16;
     // register budget of every chunk function: 64 lets one block of 32 warps fill
-    // an SM (configuration 5, 2^19 subdomains: 72 registers and 28 warps 55 ms, 80
-    // and 24 60 ms, 128 and 16 67 ms; as two blocks of 8 warps, which stream
-    // through the code separately, 82 ms)
+    // an SM (configuration 5, 2^19 subdomains: 48.9 ms; 72 registers and 28 warps 48.8, 80
+    // and 24 52.9, 128 and 16 58.9; as two blocks of 16 warps, which stream
+    // through the code separately, 64.6; configuration 2 2.05 ms, 128 and 2 x 8 warps 2.68)
     int max_regs = 64;
-    int ilp = 1;                 // subdomains per thread (1, or 2 interleaved)
+    // subdomains per thread: 2 interleaved take 58.7 ms on configuration 5 (69.3 with 128
+    // registers and half the threads), 2.66 on configuration 2 (3.07)
+    int ilp = 1;
     // short interval operations out of line: 0 none, 1 all, 2 products only (a
-    // call costs more than the two instructions of a sum: configuration 5 56 ms
-    // against 57 with 1, configuration 3 8.8 against 9.0, and 9.6 with 0)
+    // call costs more than the two instructions of a sum: configuration 5 48.9 ms
+    // against 51.4 with 1 and 53.9 with 0, configuration 3 7.84 against 8.01 and 8.48)
     int outline = 2;
 };
 struct SegSource {
