@@ -531,8 +531,8 @@ KERNEL_SOURCES = {
                     "ivb_emu.cuh"),
     "specialised": ("ivb_jit.cpp", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fixed.cuh", "ivb_fp64x.cuh",
                     "ivb_emu.cuh"),
-    "segmented": ("ivb_jit_seg.cpp", "ivb_jit.h", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fixed.cuh", "ivb_fp64x.cuh",
-                    "ivb_emu.cuh"),
+    "segmented": ("ivb_jit_seg.cpp", "ivb_jit.h", "ivb_launch.h", "ivb_bound_common.cuh", "ivb_iv.cuh", "ivb_fixed.cuh",
+                  "ivb_fp64x.cuh", "ivb_emu.cuh"),
 }
 
 
