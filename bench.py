@@ -98,7 +98,7 @@ def workload_desc(nodes, world):
                         "= 2^24 subdomains x 11 outputs",
             "nodes_per_step_per_gpu": nodes, "subdomains_per_node": 1 << 18, "outputs": 11,
             "gradients": "adjoint (reverse-mode interval)", "launch": "one persistent launch per step, CUDA graph",
-            "l2": "flushed between timed steps (256 MiB write); the kernel's state area (~0.3-0.9 GB) exceeds L2",
+            "l2": "flushed between timed steps (256 MiB write); the kernel's state area (about 1 GB) exceeds L2",
             "parallelism": f"nodes sharded over {world} GPU(s)"}
 
 
@@ -419,7 +419,8 @@ def roofline_block(p, subs_step, step_s, clk, dev, probes=False, tape=None):
     seg = p.get_segmentation()
     which = {0: "interpreter", 1: "specialised", 2: "segmented"}[p.get_tuning()["kernel"]]
     rf = {"bound": "alu", "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "G FP64 endpoint-op/s",
-          "frac": achieved / peak, "traffic": traffic_for(subs_step, which),
+          "frac": achieved / peak, "frac_note": "operations on the integer pipes included: pipe_busy_frac is the utilisation",
+          "traffic": traffic_for(subs_step, which),
           "peak_source": f"derived: {sms} SMs x 2 FP64 lanes/clock x {clock_mhz:.0f} MHz (SM clock sampled during "
                          f"the steps) = {2 * peak / 1e12:.3f} FP64 TFLOP/s; MEASURED_PEAKS.json has no FP64 figure",
           "work_per_subdomain": {"endpoint_ops": ops_per_sub, "counts": counts,
